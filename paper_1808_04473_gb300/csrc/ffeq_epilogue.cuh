@@ -46,4 +46,35 @@ __device__ __forceinline__ void symbol_llr(float2 z, float s2, float scale, int 
   }
 }
 
+// symbol_llr with the stores as wide as the address allows (the buffer itself is
+// only promised to be 4-byte aligned).  For the epilogues that walk padded
+// outputs; the exact-width solve and the batch measured 1-1.6% slower with it.
+template <int H>
+__device__ __forceinline__ void symbol_llr_h(float2 z, float inv, float scale, float* out) {
+  float v[2 * H];
+  axis_llr<H>(z.x, inv, scale, v);
+  axis_llr<H>(z.y, inv, scale, v + H);
+  if (H % 2 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+#pragma unroll
+    for (int t = 0; t + 3 < 2 * H; t += 4)
+      *reinterpret_cast<float4*>(out + t) = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+  } else if ((reinterpret_cast<uintptr_t>(out) & 7) == 0) {
+#pragma unroll
+    for (int t = 0; t < 2 * H; t += 2) *reinterpret_cast<float2*>(out + t) = make_float2(v[t], v[t + 1]);
+  } else {
+#pragma unroll
+    for (int t = 0; t < 2 * H; ++t) out[t] = v[t];
+  }
+}
+
+__device__ __forceinline__ void symbol_llr_wide(float2 z, float s2, float scale, int h, float* out) {
+  const float inv = isinf(s2) ? 0.f : rcp_approx(s2);   // s2 = 0: +inf; NaN stays NaN
+  switch (h) {
+    case 1: symbol_llr_h<1>(z, inv, scale, out); break;
+    case 2: symbol_llr_h<2>(z, inv, scale, out); break;
+    case 3: symbol_llr_h<3>(z, inv, scale, out); break;
+    default: symbol_llr_h<4>(z, inv, scale, out); break;
+  }
+}
+
 }  // namespace ffeq

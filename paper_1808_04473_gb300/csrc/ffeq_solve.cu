@@ -4,16 +4,13 @@
 // D = [G ; (y^MRC)^T] of (U + n_sym) x U complex per (subcarrier, cluster):
 // G[u][v] = D[v][u], y^MRC_u(n) = D[U+n][u].  Column i of D is therefore row i of
 // the augmented system [G + rho I | y^MRC] (rho = N0/Es, Sec. III-A), up to the
-// added rho.  One group of UP lanes (UP = U padded to 8/16/32; lane i = user i)
-// keeps its row in registers and runs a Gauss-Jordan sweep: at step k the pivot
-// row is scaled by 1/p_k, broadcast through shared memory, and eliminated from
-// every other row, while the pivot column is replaced by the inverse.  After U
-// steps the left block holds A = (G + rho I)^{-1} and the right block holds
-// z = A y^MRC for all n_sym right-hand sides.  The pivots p_k are the Schur
-// complements of the Hermitian positive definite matrix, i.e. the squared
+// added rho.  A group of lanes runs a Gauss-Jordan sweep on it: one lane per row
+// where U fills the group (8, 16 or 32) and in batches (ffeq_gj.cuh: A = (G +
+// rho I)^{-1}, then z = A y^MRC per right-hand side), else register tiles of the
+// augmented system padded to a multiple of 8 users (ffeq_tile.cuh: the right-hand
+// sides are swept along).  The pivots p_k are the Schur complements of the Hermitian positive definite matrix, i.e. the squared
 // diagonal of its Cholesky factor: a pivot that is not positive marks a failed
-// factorization at the same index k.  Every lane does the same (U + n_sym)
-// complex updates per step (no triangular idle lanes).
+// factorization at the same index k.
 //
 // A CTA holds the C clusters of one subcarrier (FD) or several subcarriers (PD)
 // and fuses per user with the optimal weights (Eq. fusionrule, Lemma 1):
@@ -32,6 +29,7 @@
 #include "ffeq_epilogue.cuh"
 #include "ffeq_gj.cuh"
 #include "ffeq_internal.h"
+#include "ffeq_tile.cuh"
 
 namespace ffeq {
 namespace {
@@ -150,77 +148,170 @@ __device__ void batch_epilogue(const SolveParams& p, const float2* base, const i
 // sums the Ceff fusion numerators and denominators of its subcarrier and writes
 // z = num / den, sigma^2 = s2_scale / den (s2_scale = N0 for the solve, whose
 // denominators are g / A_uu; Es for MRC, whose are Es / sigma_c^2) and the LLRs.
-// zflag [spc][UP] (MRC, or nullptr): users fused with the N0 -> 0 limit weights,
-// whose variance is 0.
+// System m's fusion area (numerators [n][UP], denominators) is areas + m stride.
+// Outputs are walked in the padded order (n, u < UP), so that the index splits
+// by a constant.  zflag [spc][UP] (MRC, or nullptr): users fused with the
+// N0 -> 0 limit weights, whose variance is 0.
 template <int UP>
-__device__ __forceinline__ void uniform_epilogue(const SolveParams& p, const float2* base, const int* fail_sc,
-                                                 int sc0, int U, int NS, int Ceff, float s2_scale,
+__device__ __forceinline__ void uniform_epilogue(const SolveParams& p, const float2* areas, int stride,
+                                                 const int* fail_sc, int sc0, int U, int NS, int Ceff, float s2_scale,
                                                  const int* zflag = nullptr) {
-  using Lay = SolveLayout<UP>;
-  const int spc = p.spc;
-  const int per = U * NS;   // uniform problem: every group has the problem's sizes
   const int bits = p.llr_bits, hb = bits / 2;
-  for (int e = threadIdx.x; e < spc * per; e += blockDim.x) {
-    const int s = e / per, r = e - s * per;
-    const int n = r / U, u = r - n * U;
+  for (int s = 0; s < p.spc; ++s) {
     const int k = sc0 + s;
     if (k >= p.n_sc) break;
-    float2 nm = make_float2(0.f, 0.f);
-    float dn = 0.f;
-    for (int cc = 0; cc < Ceff; ++cc) {
-      const float2* Lm = base + (s * Ceff + cc) * Lay::kMat + Lay::kRow;
-      nm = cadd(nm, Lm[n * UP + u]);
-      dn += reinterpret_cast<const float*>(Lm + Lay::kNum)[u];
+    const float2* sys = areas + static_cast<size_t>(s) * Ceff * stride;
+    const bool failed = fail_sc[s] != 0;
+    for (int e = threadIdx.x; e < UP * NS; e += blockDim.x) {
+      const int n = e / UP, u = e % UP;
+      if (u >= U) continue;
+      float2 nm = make_float2(0.f, 0.f);
+      float dn = 0.f;
+      for (int cc = 0; cc < Ceff; ++cc) {
+        nm = cadd(nm, sys[cc * stride + e]);
+        dn += reinterpret_cast<const float*>(sys + cc * stride + kNsymMax * UP)[u];
+      }
+      float2 zz;
+      float s2;
+      if (failed) {
+        zz = make_float2(NAN, NAN);
+        s2 = NAN;
+      } else if (dn > 0.f) {
+        const float rr = rcp_approx(dn);
+        zz = cscale(nm, rr);
+        s2 = (zflag && zflag[s * UP + u]) ? 0.f : s2_scale * rr;
+      } else {
+        zz = make_float2(0.f, 0.f);
+        s2 = INFINITY;
+      }
+      const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
+      p.z[zi] = zz;
+      if (n == 0) p.sigma2[static_cast<size_t>(k) * U + u] = s2;
+      if (bits) symbol_llr_wide(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
     }
-    float2 zz;
-    float s2;
-    if (fail_sc[s]) {
-      zz = make_float2(NAN, NAN);
-      s2 = NAN;
-    } else if (dn > 0.f) {
-      const float rr = rcp_approx(dn);
-      zz = cscale(nm, rr);
-      s2 = (zflag && zflag[s * UP + u]) ? 0.f : s2_scale * rr;
-    } else {
-      zz = make_float2(0.f, 0.f);
-      s2 = INFINITY;
-    }
-    const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
-    p.z[zi] = zz;
-    if (n == 0) p.sigma2[static_cast<size_t>(k) * U + u] = s2;
-    if (bits) symbol_llr(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
   }
 }
 
-// LPR lanes per row: with LPR = 2 the two lanes of row i hold halves of its
-// augmented row (columns [0, W/2) and [W/2, W)), halving the work per lane and
-// step; the pivot column k < UP always lies in the first half.
-// Uniform problems with one lane per row and up to 16 users: at most 64
-// registers, so that 8 CTAs of 128 threads fit one SM (the FD throughput
-// workload's 1200 subcarriers then run in one wave).
-template <int UP, int LPR, bool BATCH>
-constexpr int solve_min_blocks() {
-  return (!BATCH && LPR == 1 && UP <= 16) ? 2 : 1;
+// Shared memory of the uniform kernel: failure flags (256 bytes), one sweep
+// buffer per lane group, one fusion area per system.
+template <int UP>
+struct TileSolveLayout {
+  static constexpr int kArea = ((kNsymMax * UP + UP / 2 + 15) / 16) * 16 + 2;   // float2 (16-byte multiples)
+  static size_t bytes(int groups, int systems) {
+    return 256 + static_cast<size_t>(groups) * tile_smem_floats(UP) * 4 + static_cast<size_t>(systems) * kArea * 8;
+  }
+};
+
+// Uniform problems: a CTA solves the spc Ceff systems of its spc subcarriers
+// (FD: the C clusters of one subcarrier; PD: several subcarriers), a lane group
+// at a time where there are more systems than groups, fuses and writes the
+// outputs.
+template <int UP, int NRC, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 128 ? (UP <= 16 ? 5 : 3) : 1) solve_tile_kernel(const SolveParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  using Lay = TileSolveLayout<UP>;
+  constexpr int GL = TileShape<UP, NRC>::GL;
+  const int U = p.U, NS = p.n_sym, Ceff = p.Ceff, spc = p.spc;
+  const int nmat = spc * Ceff, ngrp = static_cast<int>(blockDim.x) / GL;
+  const int grp = threadIdx.x / GL, gl = threadIdx.x % GL;
+  const bool lane_ok = gl < UP;
+  const int r = lane_ok ? gl / 4 : UP / 4 - 1, q = gl % 4;
+  int* fail_sc = reinterpret_cast<int*>(smem);                     // [spc]
+  float* buf = reinterpret_cast<float*>(smem + 256) + grp * tile_smem_floats(UP);
+  float2* areas = reinterpret_cast<float2*>(smem + 256 + static_cast<size_t>(ngrp) * tile_smem_floats(UP) * 4);
+  const int sc0 = blockIdx.x * spc;
+  if (threadIdx.x < 64) fail_sc[threadIdx.x] = 0;
+  __syncthreads();
+  // Wait for the contraction grid (programmatic dependent launch).
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  const size_t mat = static_cast<size_t>(U + NS) * U;
+  for (int m0 = 0; m0 < nmat; m0 += ngrp) {
+    const int m = m0 + grp;
+    const int scl = m / Ceff, c = m - scl * Ceff;
+    const int sc = sc0 + scl;
+    const bool live = m < nmat && sc < p.n_sc;
+    const size_t sys = static_cast<size_t>(live ? sc : 0) * Ceff + (live ? c : 0);
+    float2* Fz = areas + static_cast<size_t>(m < nmat ? m : 0) * Lay::kArea;
+    const int fail = tile_solve_system<UP, NRC>(p.D + sys * mat, U, NS, p.rho, p.unbiased, live, lane_ok && m < nmat, r, q,
+                                           buf, Fz, reinterpret_cast<float*>(Fz + kNsymMax * UP),
+                                           p.Xs ? p.Xs + sys * NS * U : nullptr, p.Xs ? p.As + sys * U * U : nullptr);
+    if (gl == 0 && live) {
+      if (p.info) p.info[sys] = fail;
+      if (p.Xs) p.fails[sys] = fail;
+      else if (fail) atomicOr(&fail_sc[scl], 1);
+    }
+  }
+  if (p.Xs) return;   // the refinement kernel fuses and writes the outputs
+  __syncthreads();
+  uniform_epilogue<UP>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
 }
 
-template <int UP, int LPR, bool BATCH>
-__global__ void __launch_bounds__(512, (solve_min_blocks<UP, LPR, BATCH>())) solve_fuse_kernel(const SolveParams p) {
+template <int UP, int NRC, int MAXT>
+cudaError_t launch_tile(const SolveParams& base, cudaStream_t stream) {
+  constexpr int GL = TileShape<UP, NRC>::GL;
+  SolveParams p = base;
+  // A CTA of at least a warp: several subcarriers where one has fewer lanes.
+  p.spc = p.Ceff * GL < 32 ? 32 / (p.Ceff * GL) : 1;
+  const int nmat = p.spc * p.Ceff;
+  int threads = ((nmat * GL + 31) / 32) * 32;
+  if (threads > MAXT) threads = MAXT;
+  const size_t smem = TileSolveLayout<UP>::bytes(threads / GL, nmat);
+  static int configured[64] = {0};
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if (dev < 64 && !configured[dev]) {
+    err = cudaFuncSetAttribute(solve_tile_kernel<UP, NRC, MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (err != cudaSuccess) return err;
+    configured[dev] = 1;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((p.n_sc + p.spc - 1) / p.spc);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, solve_tile_kernel<UP, NRC, MAXT>, p);
+}
+
+// CTAs of up to 128 threads, which leave the registers the tiles want (UP <= 16:
+// 5 CTAs per SM, else 3) and take the systems of a subcarrier a group at a time;
+// where every subcarrier has its own SM anyway, one wide CTA takes them at once.
+template <int UP, int NRC>
+cudaError_t launch_tile_nrc(const SolveParams& p, cudaStream_t stream) {
+  constexpr int kSms = 152;
+  if (p.Ceff * TileShape<UP, NRC>::GL > 128 && p.n_sc <= kSms) return launch_tile<UP, NRC, 512>(p, stream);
+  return launch_tile<UP, NRC, 128>(p, stream);
+}
+
+template <int UP>
+cudaError_t launch_tile_up(const SolveParams& p, cudaStream_t stream) {
+  if (p.n_sym <= 4) return launch_tile_nrc<UP, 1>(p, stream);
+  if (p.n_sym <= 8) return launch_tile_nrc<UP, 2>(p, stream);
+  return launch_tile_nrc<UP, 4>(p, stream);
+}
+
+// The tiles of an uneven batch: one group of UP LPR lanes per local system, the
+// descriptor and cluster of each slot decoded and checked here.  LPR = 1: one
+// lane per row (ffeq_gj.cuh; the tile sweep measured slower here: 421 against
+// 387 us for 4096 instances of 4 to 32 users, FD).  LPR = 2 (a tuning choice):
+// two lanes per row, each with half of its augmented row (columns [0, W/2) and
+// [W/2, W)).
+template <int UP, int LPR>
+__global__ void __launch_bounds__(512, 1) solve_batch_kernel(const SolveParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Lay = SolveLayout<UP>;
   constexpr int GS = UP * LPR;                // lanes per matrix
-  constexpr int W = UP + kNsymMax;            // augmented row width (RHS columns beyond n_sym unused)
-  constexpr int WH = W / LPR;                 // columns per lane
-  static_assert(UP <= WH, "pivot columns must lie in the first half of a row");
-  const int spc = p.spc;
-  constexpr bool batch = BATCH;
-  const int nmat = batch ? static_cast<int>(blockDim.x) / GS : spc * p.Ceff;
+  const int nmat = static_cast<int>(blockDim.x) / GS;
   const int g = threadIdx.x / GS, gl = threadIdx.x % GS;
-  const int i = gl % UP;
-  const int h = LPR == 1 ? 0 : gl / UP;        // which half of the row this lane holds
-  int* fail_sc = reinterpret_cast<int*>(smem);                       // [spc] or [tile count]
-  // Batch mode: descriptor cache for the epilogue after the flags.
-  float2* base = reinterpret_cast<float2*>(smem + 256 + (BATCH ? kEpiCacheBytes + 16 : 0));
-  const int sc0 = blockIdx.x * spc;
+  int* fail_sc = reinterpret_cast<int*>(smem);                       // [tile count]
+  // Descriptor cache for the epilogue after the flags.
+  float2* base = reinterpret_cast<float2*>(smem + 256 + kEpiCacheBytes + 16);
 
   if (threadIdx.x < 64) fail_sc[threadIdx.x] = 0;
   __syncthreads();
@@ -228,49 +319,35 @@ __global__ void __launch_bounds__(512, (solve_min_blocks<UP, LPR, BATCH>())) sol
   // Wait for the contraction grid (programmatic dependent launch).
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // ---- the system this lane group solves
-  const int gm = g < nmat ? g : nmat - 1;       // spare lanes shadow the last matrix
-  int U, NS, Ceff, scl, c, sc = 0;
-  float rho;
-  bool valid;
-  const float2* Dg;
-  int* info_at = nullptr;
-  if constexpr (!batch) {
-    U = p.U; NS = p.n_sym; Ceff = p.Ceff; rho = p.rho;
-    scl = gm / Ceff; c = gm % Ceff;
-    sc = sc0 + scl;
-    valid = g < nmat && sc < p.n_sc;
-    const size_t matSize = static_cast<size_t>(U + NS) * U;
-    Dg = p.D + (static_cast<size_t>(valid ? sc : 0) * Ceff + c) * matSize;
-    if (p.info) info_at = p.info + static_cast<size_t>(sc) * Ceff + c;
-  } else {
-    // Slot g of this tile: cluster c of its descriptor j (map checked against the tile and the buffers).
-    const SolveTile tile = p.tiles[blockIdx.x];
-    const unsigned m = g < kTileSlots ? p.slot_map[static_cast<size_t>(blockIdx.x) * kTileSlots + g] : 0xffffu;
-    const int j = static_cast<int>(m >> 8);
-    c = static_cast<int>(m & 0xffu);
-    scl = j;
-    const int dj = tile.first + j;
-    valid = m != 0xffffu && j < tile.count && j < kTileSlots && tile.first >= 0 && dj < p.n_desc;
-    const BatchDesc* d = valid ? p.desc + dj : p.desc;
-    U = d->U; NS = d->n_sym; Ceff = d->Ceff; rho = d->rho;
-    valid = valid && U >= 1 && U <= UP && NS >= 1 && NS <= kNsymMax && Ceff >= 1 && Ceff <= kTileSlots && c < Ceff;
-    const long long matSize = valid ? static_cast<long long>(U + NS) * U : 0;
-    valid = valid && span_ok(d->d_off, Ceff * matSize, p.lim.d) &&
-            (!p.info || span_ok(d->info_off, Ceff, p.lim.info));
-    if (!valid) {
-      U = UP; NS = 1; Ceff = 1; c = 0; rho = 1.f;
-      if (m != 0xffffu && gl == 0 && p.status) atomicExch(p.status, FFEQ_ERR_INVALID_ARG);
-    }
-    Dg = p.D + (valid ? d->d_off + c * matSize : 0);
-    if (p.info && valid) info_at = p.info + d->info_off + c;
+  // Slot g of this tile: cluster c of its descriptor j (map checked against the tile and the buffers).
+  const SolveTile tile = p.tiles[blockIdx.x];
+  const unsigned m = g < kTileSlots ? p.slot_map[static_cast<size_t>(blockIdx.x) * kTileSlots + g] : 0xffffu;
+  const int j = static_cast<int>(m >> 8);
+  int c = static_cast<int>(m & 0xffu);
+  const int scl = j;
+  const int dj = tile.first + j;
+  bool valid = m != 0xffffu && j < tile.count && j < kTileSlots && tile.first >= 0 && dj < p.n_desc;
+  const BatchDesc* d = valid ? p.desc + dj : p.desc;
+  int U = d->U, NS = d->n_sym, Ceff = d->Ceff;
+  float rho = d->rho;
+  valid = valid && U >= 1 && U <= UP && NS >= 1 && NS <= kNsymMax && Ceff >= 1 && Ceff <= kTileSlots && c < Ceff;
+  const long long matSize = valid ? static_cast<long long>(U + NS) * U : 0;
+  valid = valid && span_ok(d->d_off, Ceff * matSize, p.lim.d) &&
+          (!p.info || span_ok(d->info_off, Ceff, p.lim.info));
+  if (!valid) {
+    U = UP; NS = 1; Ceff = 1; c = 0; rho = 1.f;
+    if (m != 0xffffu && gl == 0 && p.status) atomicExch(p.status, FFEQ_ERR_INVALID_ARG);
   }
-  float2* rowbuf = base + gm * Lay::kMat;
+  const float2* Dg = p.D + (valid ? d->d_off + c * matSize : 0);
+  int* info_at = nullptr;
+  if (p.info && valid) info_at = p.info + d->info_off + c;
+  float2* rowbuf = base + (g < nmat ? g : nmat - 1) * Lay::kMat;   // spare lanes shadow the last slot
   float2* Fz = rowbuf + Lay::kRow;
   float* Dn = reinterpret_cast<float*>(Fz + Lay::kNum);
 
   int fail = 0;
   if constexpr (LPR == 1) {
+    const int i = gl;
     // ---- row i of G + rho I in registers (padding: identity); the right-hand
     // sides y^MRC go straight to this system's shared block ys[n][u] (the fusion
     // terms overwrite it later).  Loads are unconditional where the address is
@@ -281,23 +358,14 @@ __global__ void __launch_bounds__(512, (solve_min_blocks<UP, LPR, BATCH>())) sol
 #pragma unroll
     for (int j = 0; j < UP; ++j) {
       const int row = j < U ? j : 0;
-      if constexpr (batch) {
-        mrow[j] = valid ? Dg[row * U + ic] : make_float2(0.f, 0.f);
-      } else {
-        mrow[j] = Dg[row * U + ic];   // invalid groups read subcarrier 0 (in bounds)
-      }
+      mrow[j] = valid ? Dg[row * U + ic] : make_float2(0.f, 0.f);
     }
     if (g < nmat) {
 #pragma unroll
       for (int n = 0; n < kNsymMax; ++n) {
         const bool real = valid && i < U && n < NS;
         float2 v = make_float2(0.f, 0.f);
-        if constexpr (batch) {
-          if (real) v = Dg[(U + n) * U + ic];
-        } else {
-          v = Dg[(real ? U + n : 0) * U + ic];
-          if (!real) v = make_float2(0.f, 0.f);
-        }
+        if (real) v = Dg[(U + n) * U + ic];
         ys[n * UP + i] = v;
       }
     }
@@ -339,12 +407,6 @@ __global__ void __launch_bounds__(512, (solve_min_blocks<UP, LPR, BATCH>())) sol
     // mu = [A G]_ii = 1 - rho A_ii; a user the cluster cannot see (G_ii = 0) has
     // mu = 0 exactly, which the subtraction would only reach up to rounding.
     const float mu = gii == 0.f ? 0.f : fmaxf(1.f - rho * Ai, 0.f);
-    bool store = false;
-    size_t sys = 0;
-    if constexpr (!batch) {
-      store = p.Xs != nullptr;   // refinement follows: keep estimates and inverses
-      sys = static_cast<size_t>(sc) * Ceff + c;
-    }
     // z_n = sum_j A[i][j] y^MRC_j(n) in j order; after every lane of the warp has
     // read row n of ys, the fusion term z_n / A_ii replaces it ([n][u]: the
     // epilogue reads along u).
@@ -360,186 +422,113 @@ __global__ void __launch_bounds__(512, (solve_min_blocks<UP, LPR, BATCH>())) sol
         }
       }
       __syncwarp();
-      if (n < NS && g < nmat) {
-        if (store) {
-          if (valid && i < U) p.Xs[(sys * NS + n) * U + i] = zn;
-        } else {
-          ys[n * UP + i] = cscale(zn, invA);
-        }
-      }
+      if (n < NS && g < nmat) ys[n * UP + i] = cscale(zn, invA);
     }
-    if (store) {
-      // Inverse stored transposed (row j = column j of A, coalesced over the lanes i).
-      if (g < nmat && valid && i < U) {
-#pragma unroll
-        for (int j = 0; j < UP; ++j)
-          if (j < U) p.As[(sys * U + j) * U + i] = arow[j];
-        if (gl == 0) {
-          p.fails[sys] = fail;
-          if (info_at) *info_at = fail;
-        }
-      }
-      return;   // the refinement kernel fuses and writes the outputs
-    }
-    if (g < nmat) {
-      Dn[i] = (p.unbiased ? mu : 1.f) * invA;
-      if (gl == 0 && valid) {
-        if (info_at) *info_at = fail;
-        if (fail) atomicOr(&fail_sc[scl], 1);
-      }
-    }
+    if (g < nmat) Dn[i] = (p.unbiased ? mu : 1.f) * invA;
   } else {
-    // ---- this lane's columns of row i of [G + rho I | y^MRC] (padding: identity, zero RHS)
-    // Loads are unconditional (clamped to valid addresses) so they all issue before
-    // the first use; padding values are selected afterwards.
+    const int i = gl % UP;
+    const int h = gl / UP;                     // which half of the row this lane holds
+    constexpr int W = UP + kNsymMax;           // augmented row width (right-hand sides beyond n_sym unused)
+    constexpr int WH = W / LPR;                // columns per lane
+    static_assert(UP <= WH, "pivot columns must lie in the first half of a row");
+    // This lane's columns of row i of [G + rho I | y^MRC] (padding: identity, zero).
     float2 aug[WH];
     const int ic = i < U ? i : 0;
-  #pragma unroll
-    for (int j = 0; j < WH; ++j) {
-      const int col = h * WH + j;
+#pragma unroll
+    for (int jj = 0; jj < WH; ++jj) {
+      const int col = h * WH + jj;
       const int row = col < UP ? (col < U ? col : 0) : (col - UP < NS ? U + col - UP : 0);
-      if constexpr (batch) {
-        aug[j] = valid ? Dg[row * U + ic] : make_float2(0.f, 0.f);
-      } else {
-        aug[j] = Dg[row * U + ic];   // invalid groups read subcarrier 0 (in bounds)
-      }
+      aug[jj] = valid ? Dg[row * U + ic] : make_float2(0.f, 0.f);
     }
     float gii = 1.f;
-  #pragma unroll
-    for (int j = 0; j < WH; ++j) {
-      const int col = h * WH + j;
+#pragma unroll
+    for (int jj = 0; jj < WH; ++jj) {
+      const int col = h * WH + jj;
       const bool real = valid && i < U && (col < UP ? col < U : col - UP < NS);
-      float2 v = real ? aug[j] : make_float2(col == i ? 1.f : 0.f, 0.f);
+      float2 v = real ? aug[jj] : make_float2(col == i ? 1.f : 0.f, 0.f);
       if (col == i && real) {
         gii = v.x;
         v = make_float2(v.x + rho, 0.f);
       }
-      aug[j] = v;
+      aug[jj] = v;
     }
-
-      // ---- Gauss-Jordan sweep (deferred row scaling: every lane runs the same update)
-      // Two lanes per row, columns in place: the same element update as the paired
-      // form (gj_update), so both layouts give identical bits.
-      float my_r = 1.f;
-      static_for<UP>([&](auto kc) {
-        constexpr int k = decltype(kc)::value;
-        const float piv = __shfl_sync(kFullMask, aug[k].x, k, GS);
-        const float2 f = make_float2(__shfl_sync(kFullMask, aug[k].x, i, GS), __shfl_sync(kFullMask, aug[k].y, i, GS));
-        const bool ok = piv > 0.f;
-        if (!ok && fail == 0) fail = k + 1;
-        const float r = rcp_approx(ok ? piv : 1.f);
-        const bool me = i == k;
-        if (me) my_r = r;
-        const float2 gg = me ? make_float2(0.f, 0.f) : make_float2(f.x * r, f.y * r);
-        if (me && g < nmat) {
-  #pragma unroll
-          for (int j = 0; j < WH; j += 2)
-            if (h * WH + j < UP + NS)
-              *reinterpret_cast<float4*>(rowbuf + h * WH + j) =
-                  make_float4((h == 0 && j == k) ? 1.f : aug[j].x, (h == 0 && j == k) ? 0.f : aug[j].y,
-                              (h == 0 && j + 1 == k) ? 1.f : aug[j + 1].x, (h == 0 && j + 1 == k) ? 0.f : aug[j + 1].y);
-        }
-        __syncwarp();
-        const float dlt = me ? 1.f : 0.f;
-        const float2* rb = rowbuf + h * WH;
-  #pragma unroll
-        for (int j = 0; j < WH; j += 2) {
-          if (h * WH + j < UP + NS) {
-            const float4 q = *reinterpret_cast<const float4*>(rb + j);
-            const float2 b0 = (h == 0 && j == k) ? make_float2(dlt, 0.f) : aug[j];
-            const float2 b1 = (h == 0 && j + 1 == k) ? make_float2(dlt, 0.f) : aug[j + 1];
-            aug[j] = gj_update(gg, make_float2(q.x, q.y), b0);
-            aug[j + 1] = gj_update(gg, make_float2(q.z, q.w), b1);
-          }
-        }
-        __syncwarp();
-      });
-      // Deferred scaling: row i times 1/p_i (both halves of row i recorded it at step i).
-  #pragma unroll
-      for (int j = 0; j < WH; ++j) aug[j] = cscale(aug[j], my_r);
-
-    if constexpr (!batch) {
-      if (p.Xs) {
-        // Refinement follows: keep this system's estimates X [n][u] and its inverse
-        // stored transposed (row j = column j of A, coalesced over the lanes i).
-        if (g < nmat && valid && i < U) {
-          const size_t sys = static_cast<size_t>(sc) * Ceff + c;
-  #pragma unroll
-          for (int j = 0; j < WH; ++j) {
-            if constexpr (LPR == 1) {
-              if (j >= kNsymMax && j - kNsymMax < U) p.As[(sys * U + (j - kNsymMax)) * U + i] = aug[j];
-              if (j < NS) p.Xs[(sys * NS + j) * U + i] = aug[j];
-            } else {
-              const int col = h * WH + j;
-              if (col < U) p.As[(sys * U + col) * U + i] = aug[j];
-              if (col >= UP && col - UP < NS) p.Xs[(sys * NS + (col - UP)) * U + i] = aug[j];
-            }
-          }
-          if (gl == 0) {
-            p.fails[sys] = fail;
-            if (info_at) *info_at = fail;
-          }
-        }
-        return;   // the refinement kernel fuses and writes the outputs
+    // Gauss-Jordan sweep, deferred row scaling, columns in place.
+    float my_r = 1.f;
+    static_for<UP>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      const float piv = __shfl_sync(kFullMask, aug[k].x, k, GS);
+      const float2 f = make_float2(__shfl_sync(kFullMask, aug[k].x, i, GS), __shfl_sync(kFullMask, aug[k].y, i, GS));
+      const bool ok = piv > 0.f;
+      if (!ok && fail == 0) fail = k + 1;
+      const float rc = rcp_approx(ok ? piv : 1.f);
+      const bool me = i == k;
+      if (me) my_r = rc;
+      const float2 gg = me ? make_float2(0.f, 0.f) : make_float2(f.x * rc, f.y * rc);
+      if (me) {
+#pragma unroll
+        for (int jj = 0; jj < WH; jj += 2)
+          if (h * WH + jj < UP + NS)
+            *reinterpret_cast<float4*>(rowbuf + h * WH + jj) =
+                make_float4((h == 0 && jj == k) ? 1.f : aug[jj].x, (h == 0 && jj == k) ? 0.f : aug[jj].y,
+                            (h == 0 && jj + 1 == k) ? 1.f : aug[jj + 1].x, (h == 0 && jj + 1 == k) ? 0.f : aug[jj + 1].y);
       }
-    }
-
-    // ---- fusion terms of this matrix: A_ii on the first-half lane of row i
-    // (column i before rotation; column kNsymMax + i after the rotating sweep)
-    constexpr int kA = LPR == 1 ? kNsymMax : 0;   // first column of A in this lane's registers
-    constexpr int kZ = LPR == 1 ? 0 : UP;         // first RHS column (global column index)
+      __syncwarp();
+      const float dlt = me ? 1.f : 0.f;
+      const float2* rb = rowbuf + h * WH;
+#pragma unroll
+      for (int jj = 0; jj < WH; jj += 2) {
+        if (h * WH + jj < UP + NS) {
+          const float4 qv = *reinterpret_cast<const float4*>(rb + jj);
+          const float2 b0 = (h == 0 && jj == k) ? make_float2(dlt, 0.f) : aug[jj];
+          const float2 b1 = (h == 0 && jj + 1 == k) ? make_float2(dlt, 0.f) : aug[jj + 1];
+          aug[jj] = gj_update(gg, make_float2(qv.x, qv.y), b0);
+          aug[jj + 1] = gj_update(gg, make_float2(qv.z, qv.w), b1);
+        }
+      }
+      __syncwarp();
+    });
+    // Deferred scaling: row i times 1/p_i (both halves of row i recorded it at step i).
+#pragma unroll
+    for (int jj = 0; jj < WH; ++jj) aug[jj] = cscale(aug[jj], my_r);
+    // Fusion terms of this matrix: A_ii on the first-half lane of row i.
     float Ai = 1.f;
-  #pragma unroll
-    for (int j = 0; j < UP; ++j)
-      if (j == i) Ai = aug[kA + j].x;
+#pragma unroll
+    for (int jj = 0; jj < UP; ++jj)
+      if (jj == i) Ai = aug[jj].x;
     Ai = __shfl_sync(kFullMask, Ai, i, GS);
     const float invA = rcp_approx(Ai);
-    // mu = [A G]_ii = 1 - rho A_ii; a user the cluster cannot see (G_ii = 0) has
-    // mu = 0 exactly, which the subtraction would only reach up to rounding.
     const float mu = gii == 0.f ? 0.f : fmaxf(1.f - rho * Ai, 0.f);
-    if (g < nmat) {
-  #pragma unroll
-      for (int j = 0; j < WH; ++j) {
-        const int n = h * WH + j - kZ;
-        if (n >= 0 && n < NS && (LPR != 1 || j < kNsymMax))
-          Fz[n * UP + i] = cscale(aug[j], invA);   // [n][u]: the epilogue reads along u
-      }
-      if (h == 0) Dn[i] = (p.unbiased ? mu : 1.f) * invA;
-      if (gl == 0 && valid) {
-        if (info_at) *info_at = fail;
-        if (fail) atomicOr(&fail_sc[scl], 1);
-      }
+#pragma unroll
+    for (int jj = 0; jj < WH; ++jj) {
+      const int n = h * WH + jj - UP;
+      if (n >= 0 && n < NS) Fz[n * UP + i] = cscale(aug[jj], invA);   // [n][u]: the epilogue reads along u
     }
+    if (h == 0) Dn[i] = (p.unbiased ? mu : 1.f) * invA;
+  }
+  if (gl == 0 && valid && g < nmat) {
+    if (info_at) *info_at = fail;
+    if (fail) atomicOr(&fail_sc[scl], 1);
   }
   __syncthreads();
-  if constexpr (batch) {
-    batch_epilogue<UP>(p, base, fail_sc, nmat, reinterpret_cast<EpiDesc*>(smem + 256),
-                       reinterpret_cast<int*>(smem + 256 + kEpiCacheBytes));
-    return;
-  }
-
-  uniform_epilogue<UP>(p, base, fail_sc, sc0, U, NS, Ceff, p.N0);
+  batch_epilogue<UP>(p, base, fail_sc, nmat, reinterpret_cast<EpiDesc*>(smem + 256),
+                     reinterpret_cast<int*>(smem + 256 + kEpiCacheBytes));
 }
 
-template <int UP, int LPR, bool BATCH>
-cudaError_t launch_up(const SolveParams& p, cudaStream_t stream) {
-  using Lay = SolveLayout<UP>;
-  constexpr bool batch = BATCH;
-  const int nmat = batch ? p.threads / (UP * LPR) : p.spc * p.Ceff;
-  const int threads = batch ? p.threads : ((nmat * UP * LPR + 31) / 32) * 32;
-  const size_t smem = 256 + (batch ? kEpiCacheBytes + 16 : 0) + static_cast<size_t>(nmat) * Lay::kMat * sizeof(float2);
+template <int UP, int LPR>
+cudaError_t launch_batch_up(const SolveParams& p, cudaStream_t stream) {
+  const size_t smem = solve_batch_smem_bytes(UP, LPR, p.threads, p.equalizer);
   static int configured[64] = {0};
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   if (dev < 64 && !configured[dev]) {
-    err = cudaFuncSetAttribute(solve_fuse_kernel<UP, LPR, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    err = cudaFuncSetAttribute(solve_batch_kernel<UP, LPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (err != cudaSuccess) return err;
     configured[dev] = 1;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(batch ? p.n_tiles : (p.n_sc + p.spc - 1) / p.spc);
-  cfg.blockDim = dim3(threads);
+  cfg.gridDim = dim3(p.n_tiles);
+  cfg.blockDim = dim3(p.threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -547,13 +536,12 @@ cudaError_t launch_up(const SolveParams& p, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, solve_fuse_kernel<UP, LPR, BATCH>, p);
+  return cudaLaunchKernelEx(&cfg, solve_batch_kernel<UP, LPR>, p);
 }
 
 // Solve / fusion / soft outputs for uniform problems whose users fill the lane
-// group (U == UP: 8, 16 or 32), one lane per row.  The same computation as
-// solve_fuse_kernel's one-lane path, specialized so that the sizes that shape
-// the work are compile-time constants: every lane loads its row with fixed
+// group (U == UP: 8, 16 or 32), one lane per row (ffeq_gj.cuh), specialized so
+// that the sizes that shape the work are compile-time constants: every lane loads its row with fixed
 // offsets from one column pointer (no padding rows, no clamped or selected
 // addresses), the right-hand sides reach shared memory by asynchronous copies
 // that overlap the sweep, and the epilogue walks (symbol, user) outputs with
@@ -795,7 +783,7 @@ __global__ void __launch_bounds__(512) mrc_fuse_kernel(const SolveParams p) {
     Dn[i] = w;
   }
   __syncthreads();
-  uniform_epilogue<UP>(p, base, fail_sc, sc0, U, NS, Ceff, p.Es, zflag);
+  uniform_epilogue<UP>(p, base + Lay::kRow, Lay::kMat, fail_sc, sc0, U, NS, Ceff, p.Es, zflag);
 }
 
 template <int UP>
@@ -829,7 +817,7 @@ cudaError_t launch_mrc_up(const SolveParams& p, cudaStream_t stream) {
 
 // Maximum-ratio combining (Sec. III-A) for the tiles of an uneven batch: one
 // group of UP lanes per local system, the descriptor and cluster of each slot
-// decoded and checked as in solve_fuse_kernel's batch mode, the per-lane
+// decoded and checked as in solve_batch_kernel, the per-lane
 // arithmetic of mrc_fuse_kernel (weight w = Es / sigma_c^2, numerators
 // w y^MRC_i(n) / G_ii, the N0 -> 0 limit weights per descriptor with N0 = 0),
 // and the batch epilogue with sigma^2 = Es / sum w (0 for the limit-weight users).
@@ -963,20 +951,21 @@ cudaError_t launch_solve(const SolveParams& p, cudaStream_t stream) {
       default: return launch_mrc_up<32>(p, stream);
     }
   }
-  const int UP = padded_users(p.U);
-  if (p.U == UP && lanes_per_row(p.U, p.Ceff) == 1) {   // users fill the lane group
-    switch (UP) {
-      case 8: return launch_full<8>(p, stream);
-      case 16: return launch_full<16>(p, stream);
-      default: return launch_full<32>(p, stream);
-    }
+  // Users that fill a lane group: one lane per row (the tile sweep measured no
+  // faster there, 28 against 24 us for FD with U = 16, C = 8, 1200 x 14).  Any
+  // other number: the tile sweep, padded to a multiple of 8 (FD, U = 11, C = 5,
+  // 625 x 13: 32.8 -> 30.7 us a call; PD, U = 12, 333 x 7, ZF: 24.6 -> 20.5 us;
+  // against the row sweep padded to 16 or 32).
+  switch (p.U) {
+    case 8: return launch_full<8>(p, stream);
+    case 16: return launch_full<16>(p, stream);
+    case 32: return launch_full<32>(p, stream);
+    default: break;
   }
-  switch (UP) {
-    case 8: return launch_up<8, 1, false>(p, stream);
-    case 16: return lanes_per_row(p.U, p.Ceff) == 2 ? launch_up<16, 2, false>(p, stream)
-                                                    : launch_up<16, 1, false>(p, stream);
-    default: return launch_up<32, 1, false>(p, stream);
-  }
+  if (p.U < 8) return launch_tile_up<8>(p, stream);
+  if (p.U < 16) return launch_tile_up<16>(p, stream);
+  if (p.U <= 24) return launch_tile_up<24>(p, stream);
+  return launch_tile_up<32>(p, stream);
 }
 
 cudaError_t launch_solve_batch(const SolveParams& p, int lpr, cudaStream_t stream) {
@@ -989,9 +978,9 @@ cudaError_t launch_solve_batch(const SolveParams& p, int lpr, cudaStream_t strea
     }
   }
   switch (p.U) {
-    case 8: return lpr == 2 ? launch_up<8, 2, true>(p, stream) : launch_up<8, 1, true>(p, stream);
-    case 16: return lpr == 2 ? launch_up<16, 2, true>(p, stream) : launch_up<16, 1, true>(p, stream);
-    default: return launch_up<32, 1, true>(p, stream);
+    case 8: return lpr == 2 ? launch_batch_up<8, 2>(p, stream) : launch_batch_up<8, 1>(p, stream);
+    case 16: return lpr == 2 ? launch_batch_up<16, 2>(p, stream) : launch_batch_up<16, 1>(p, stream);
+    default: return launch_batch_up<32, 1>(p, stream);
   }
 }
 
