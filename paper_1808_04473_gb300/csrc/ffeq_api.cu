@@ -392,6 +392,17 @@ ffeq_status ffeq_equalize(const ffeq_plan* plan, const void* H, const void* y, f
 
 namespace {
 
+// FP32 FD problems of several clusters, in the default shape, are equalized by the
+// fused kernel where it is the faster one and a subcarrier fits one CTA's shared
+// memory (ffeq_formed.cu).
+bool formed_applies(const ffeq_plan* plan) {
+  const ffeq_problem& p = plan->p;
+  return p.precision == FFEQ_FP32 && p.refine == 0 &&
+         (p.equalizer == FFEQ_LMMSE || p.equalizer == FFEQ_ZF) &&
+         (plan->gram_variant == ffeq::kGramAuto || plan->gram_variant == ffeq::kGram16) &&
+         ffeq::equalize_formed_fits(p.B, p.U, p.n_sym, plan->Ceff, p.n_sc);
+}
+
 ffeq_status equalize_impl(const ffeq_plan* plan, const void* H, const void* y, float N0, float Es, void* z,
                           float* sigma2, float* llr, int* info, void* workspace, size_t workspace_bytes,
                           void* stream, bool host_inputs) {
@@ -419,6 +430,20 @@ ffeq_status equalize_impl(const ffeq_plan* plan, const void* H, const void* y, f
       const cudaError_t e = ffeq::launch_gram_fused(gp, sp, p.precision, st);
       return e == cudaSuccess ? FFEQ_OK : cuda_fail(e);
     }
+  }
+  if (formed_applies(plan)) {
+    // One launch from the inputs to the outputs (host inputs as well: they are read
+    // once, with plain asynchronous copies).
+    ffeq::FormedParams fp{};
+    r = solve_params(plan, workspace, N0, Es, z, sigma2, llr, info, fp.s);
+    if (r != FFEQ_OK) return r;
+    fp.H = static_cast<const float2*>(H);
+    fp.y = static_cast<const float2*>(y);
+    fp.B = p.B;
+    fp.cl_uniform = plan->cl_uniform ? 1 : 0;
+    for (int c = 0; c <= plan->Ceff && !plan->cl_uniform; ++c) fp.cl_off[c] = plan->cl_off[c];
+    const cudaError_t e = ffeq::launch_equalize_formed(fp, st);
+    return e == cudaSuccess ? FFEQ_OK : cuda_fail(e);
   }
   r = local_preprocess(plan, H, y, workspace, st, host_inputs);
   if (r != FFEQ_OK) return r;

@@ -1,0 +1,192 @@
+// Fused FP32 equalization of FD problems (L-MMSE and ZF): one launch from H and y
+// to z, sigma^2 and LLRs.
+//
+// A CTA stages one subcarrier and a lane group per cluster forms [G_c + rho I |
+// y_c^MRC] in registers (Sec. II-C, ffeq_formed.cuh), sweeps it (Sec. III-A) and
+// leaves the cluster's fusion terms in shared memory; the CTA then fuses per user
+// (Eq. fusionrule, Lemma 1; Thm. 3) and writes the outputs.  Neither the local
+// Gram matrices nor the matched filters go through the workspace, and the CUDA-core
+// contraction's staging, its partial sums and the second launch are gone.
+// What bounds it: the FMA pipe (the contraction and the sweep are about 60 / 40).
+#include <cmath>
+
+#include "ffeq_device.cuh"
+#include "ffeq_epilogue.cuh"
+#include "ffeq_formed.cuh"
+#include "ffeq_internal.h"
+
+namespace ffeq {
+namespace {
+
+constexpr int kThreads = 256;   // at most
+
+template <int UP, int NRC>
+struct FormedEqLayout {
+  static constexpr int NR = 4 * NRC;
+  static constexpr int AREA = NR * UP + UP / 2;   // float2 per cluster: numerators [NR][UP], denominators [UP]
+  static int groups(int C) {
+    const int most = kThreads / FormedShape<UP>::GL;
+    return C < most ? C : most;
+  }
+  // The areas take the place of the staged rows where every cluster has a lane
+  // group (all tiles are formed before the first term is written): 62 instead of
+  // 78 KB for B = 256, U = 16, 14 symbols, three CTAs per SM instead of two.
+  __host__ __device__ static size_t areas(int B, int rows, bool at_once) {
+    return 16 + (at_once ? 0 : formed_staged_bytes(B, rows));
+  }
+  static size_t bytes(int B, int U, int n_sym, int C) {
+    const size_t rows = formed_staged_bytes(B, U + n_sym), terms = static_cast<size_t>(C) * AREA * sizeof(float2);
+    return 16 + (groups(C) == C ? (rows > terms ? rows : terms) : rows + terms);
+  }
+  static int threads(int B, int C) {
+    const int t = groups(C) * FormedShape<UP>::GL, w = B < 128 ? B : 128;
+    return (((t > w ? t : w) + 31) / 32) * 32;
+  }
+};
+
+template <int UP, int NRC>
+__global__ void __launch_bounds__(kThreads, 2) equalize_formed_kernel(const FormedParams p, int groups) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  using F = FormedShape<UP>;
+  using Lay = FormedEqLayout<UP, NRC>;
+  constexpr int NC = F::CA + NRC;
+  const int U = p.s.U, NS = p.s.n_sym, C = p.s.Ceff, B = p.B, RS = formed_stride(B);
+  const int k = blockIdx.x;
+  const float rho = p.s.rho;
+  int* failed = reinterpret_cast<int*>(smem);
+  float* Ws = reinterpret_cast<float*>(smem + 16);
+  const bool at_once = groups == C;
+  float2* areas = reinterpret_cast<float2*>(smem + Lay::areas(B, U + NS, at_once));
+  if (threadIdx.x == 0) *failed = 0;
+  formed_stage(p.H + static_cast<size_t>(k) * U * B, p.y + static_cast<size_t>(k) * NS * B, U, NS, B, Ws);
+  formed_wait();
+
+  const int grp = threadIdx.x / F::GL, gl = threadIdx.x % F::GL, r = gl / 4, q = gl % 4;
+  if ((threadIdx.x & ~31) / F::GL >= groups) {   // whole warps without a group
+    if (at_once) __syncthreads();
+  } else {
+    for (int c0 = 0; c0 < C; c0 += groups) {
+      const bool valid = grp < groups && c0 + grp < C;
+      const int c = valid ? c0 + grp : 0;
+      const int S = p.cl_uniform ? B / C : 0;
+      const int b0 = p.cl_uniform ? c * S : p.cl_off[c], b1 = p.cl_uniform ? b0 + S : p.cl_off[c + 1];
+      float re[F::RPL][NC], im[F::RPL][NC], rs[F::RPL];
+      formed_tile<UP, NRC, true>(Ws, RS, U, NS, b0, b1, r, q, valid, 0.f, re, im);
+      if (at_once) __syncthreads();   // one pass: the staged rows are no longer read
+      unsigned zero_diag = 0;   // users this cluster cannot see (G_ii = 0), one bit per row of the lane
+#pragma unroll
+      for (int i = 0; i < F::RPL; ++i) {
+        if (formed_diagonal<UP, NC>(re, i, r) == 0.f) zero_diag |= 1u << i;
+#pragma unroll
+        for (int j = 0; j < F::CA; ++j)
+          if (q + 4 * j == r + F::RL * i && valid && r + F::RL * i < U) re[i][j] += rho;
+      }
+      const int fail = formed_sweep<UP, NRC, true>(re, im, U, r, q, rs);
+      float2* Fz = areas + static_cast<size_t>(c) * Lay::AREA;
+      float* Dn = reinterpret_cast<float*>(Fz + Lay::NR * UP);
+#pragma unroll
+      for (int i = 0; i < F::RPL; ++i) {
+        const int u = r + F::RL * i;
+        const float Ai = __shfl_sync(kFullMask, formed_diagonal<UP, NC>(re, i, r) * rs[i], 4 * r + (r & 3), F::GL);
+        const float invA = rcp_approx(Ai);
+        if (valid && q == (r & 3)) {
+          // mu = [A G]_ii = 1 - rho A_ii; a user the cluster cannot see (G_ii = 0) has
+          // mu = 0 exactly, which the subtraction would only reach up to rounding.
+          const float mu = (zero_diag >> i) & 1u ? 0.f : fmaxf(1.f - rho * Ai, 0.f);
+          Dn[u] = (p.s.unbiased ? mu : 1.f) * invA;
+        }
+#pragma unroll
+        for (int j = 0; j < NRC; ++j) {
+          const int n = q + 4 * j;
+          if (valid && n < NS)
+            Fz[n * UP + u] = make_float2(re[i][F::CA + j] * rs[i] * invA, im[i][F::CA + j] * rs[i] * invA);
+        }
+      }
+      if (valid && gl == 0) {
+        if (p.s.info) p.s.info[static_cast<size_t>(k) * C + c] = fail;
+        if (fail) atomicOr(failed, 1);
+      }
+    }
+  }
+  __syncthreads();
+  const bool bad = *failed != 0;
+  const int bits = p.s.llr_bits, hb = bits / 2;
+  for (int e = threadIdx.x; e < UP * NS; e += blockDim.x) {
+    const int n = e / UP, u = e % UP;
+    if (u >= U) continue;
+    float2 nm = make_float2(0.f, 0.f);
+    float dn = 0.f;
+    for (int c = 0; c < C; ++c) {
+      nm = cadd(nm, areas[c * Lay::AREA + e]);
+      dn += reinterpret_cast<const float*>(areas + c * Lay::AREA + Lay::NR * UP)[u];
+    }
+    float2 zz;
+    float s2;
+    if (bad) {
+      zz = make_float2(NAN, NAN);
+      s2 = NAN;
+    } else if (dn > 0.f) {
+      const float rr = rcp_approx(dn);
+      zz = cscale(nm, rr);
+      s2 = p.s.N0 * rr;
+    } else {
+      zz = make_float2(0.f, 0.f);
+      s2 = INFINITY;
+    }
+    const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
+    p.s.z[zi] = zz;
+    if (n == 0) p.s.sigma2[static_cast<size_t>(k) * U + u] = s2;
+    if (bits) symbol_llr_wide(zz, s2, p.s.llr_scale, hb, p.s.llr + zi * bits);
+  }
+}
+
+template <int UP, int NRC>
+cudaError_t launch_up(const FormedParams& p, cudaStream_t stream) {
+  using Lay = FormedEqLayout<UP, NRC>;
+  const size_t smem = Lay::bytes(p.B, p.s.U, p.s.n_sym, p.s.Ceff);
+  static int configured[64] = {0};
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if (dev < 64 && !configured[dev]) {
+    err = cudaFuncSetAttribute(equalize_formed_kernel<UP, NRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (err != cudaSuccess) return err;
+    configured[dev] = 1;
+  }
+  equalize_formed_kernel<UP, NRC><<<p.s.n_sc, Lay::threads(p.B, p.s.Ceff), smem, stream>>>(p, Lay::groups(p.s.Ceff));
+  return cudaGetLastError();
+}
+
+template <int UP>
+cudaError_t launch_nrc(const FormedParams& p, cudaStream_t stream) {
+  if (p.s.n_sym <= 4) return launch_up<UP, 1>(p, stream);
+  if (p.s.n_sym <= 8) return launch_up<UP, 2>(p, stream);
+  return launch_up<UP, 4>(p, stream);
+}
+
+}  // namespace
+
+// Measured against the contraction and solve launches (us, before -> after): U = 4,
+// C = 2, S = 16, 2000 x 1: 38.8 -> 9.2; U = 8, C = 16, 3000 x 2: 112 -> 45; U = 15, C = 3,
+// S = 85, 1200 x 14: 127 -> 78; U = 16, C = 8, S = 32, 1200 x 14: 64.0 -> 61.4; U = 32,
+// C = 4, 1000 x 7: 162 -> 142.  Where it loses, the separate launches stay: tiles of 32
+// users with 16 right-hand sides spill registers (C = 16, 3300 x 14: 825 -> 1008), and
+// two or three clusters of 32 users leave too few warps per CTA for the contraction (C = 2,
+// S = 128, 300 x 14: 48 -> 72), as those of 16 users and 16 right-hand sides do where an
+// SM has less than two subcarriers (U = 16, C = 2, 64 x 14: 16.6 -> 20.6).
+bool equalize_formed_fits(int B, int U, int n_sym, int C, int n_sc) {
+  if (C < 2 || (U > 16 && (n_sym > 8 || C < 4))) return false;
+  if (U > 8 && n_sym > 8 && C < 4 && n_sc < 2 * 152) return false;
+  const int UP = padded_users(U), NRC = n_sym <= 4 ? 1 : (n_sym <= 8 ? 2 : 4);
+  return 16 + formed_staged_bytes(B, U + n_sym) + static_cast<size_t>(C) * (4 * NRC * UP + UP / 2) * 8 <= 227 * 1024;   // bytes() at most
+}
+
+cudaError_t launch_equalize_formed(const FormedParams& p, cudaStream_t stream) {
+  switch (padded_users(p.s.U)) {
+    case 8: return launch_nrc<8>(p, stream);
+    case 16: return launch_nrc<16>(p, stream);
+    default: return launch_nrc<32>(p, stream);
+  }
+}
+
+}  // namespace ffeq

@@ -136,6 +136,20 @@ struct SolveParams {
   int* fails;
 };
 
+// Fused FP32 equalization of an FD problem (ffeq_formed.cu): the solve's outputs and
+// scalars (s.D is not read) with the inputs and clusters of the contraction.
+struct FormedParams {
+  const float2* H;      // [n_sc][U][B]
+  const float2* y;      // [n_sc][n_sym][B]
+  int B;
+  SolveParams s;
+  int cl_uniform;       // B / C antennas per cluster, else cl_off
+  int cl_off[kMaxClusters + 1];
+};
+// Whether that launch applies and is the faster one.
+bool equalize_formed_fits(int B, int U, int n_sym, int C, int n_sc);
+cudaError_t launch_equalize_formed(const FormedParams& p, cudaStream_t stream);
+
 // Iterative refinement from the inputs (uniform problems).
 struct RefineParams {
   const float2* H;      // [n_sc][U][B]
