@@ -311,6 +311,7 @@ ffeq_status fuse_equalize(const ffeq_plan* plan, const void* workspace, float N0
     sp.Xs = reinterpret_cast<float2*>(ws + plan->off_X);
     sp.As = reinterpret_cast<float2*>(ws + plan->off_A);
     sp.fails = reinterpret_cast<int*>(ws + plan->off_F);
+    sp.cond = p.refine_fp64 == 1;
   }
   if (p.equalizer == FFEQ_LAMA) {
     sp.lama_iters = p.lama_iters;

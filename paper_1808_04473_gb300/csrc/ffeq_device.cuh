@@ -37,6 +37,13 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+// The hardware's approximate square root (PTX sqrt.approx.ftz.f32), for estimates.
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // ---------------------------------------------------------------- complex (float2)
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }

@@ -129,11 +129,12 @@ struct SolveParams {
   BatchLimits lim;
   int* status;
   // Uniform problem with refinement: write the local estimates X [n_sc][Ceff][n_sym][U],
-  // the inverses transposed As [n_sc][Ceff][U][U] and the pivot status fails
-  // [n_sc][Ceff] instead of the outputs.
+  // the inverses transposed As [n_sc][Ceff][U][U] and the status words fails
+  // [n_sc][Ceff] (kRefinePivotMask, kRefineFp64Mark) instead of the outputs.
   float2* Xs;
   float2* As;
   int* fails;
+  int cond;           // refinement with the FP64 residual above a condition threshold: mark the systems
 };
 
 // Fused FP32 equalization of an FD problem (ffeq_formed.cu): the solve's outputs and
@@ -150,14 +151,23 @@ struct FormedParams {
 bool equalize_formed_fits(int B, int U, int n_sym, int C, int n_sc);
 cudaError_t launch_equalize_formed(const FormedParams& p, cudaStream_t stream);
 
+// Status word of a system between the solve and its refinement (fails): the
+// 1-based failing pivot, and a mark on systems whose condition estimate
+// ||G_c + rho I||_1 ||A~_c||_1 exceeds kCondFp64 (their residual is FP64 with
+// refine_fp64 = 1).
+constexpr int kRefinePivotMask = 0xffff, kRefineFp64Mark = 1 << 16;
+constexpr float kCondFp64 = 1e4f;
+
 // Iterative refinement from the inputs (uniform problems).
 struct RefineParams {
   const float2* H;      // [n_sc][U][B]
   const float2* y;      // [n_sc][n_sym][B]
   const float2* D;      // contraction output (for G_uu)
-  float2* As;           // [n_sc][Ceff][U][U] inverses, transposed (the diagonal refined in place)
+  float2* As;           // [n_sc][Ceff][U][U] inverses, transposed; after refinement the first U
+                        // entries of a system hold (A_uu, G_uu)
   float2* Xs;           // [n_sc][Ceff][n_sym][U] (refined in place)
   const int* fails;     // [n_sc][Ceff]
+  int only64;           // the generic kernel takes the systems with the FP64 residual alone
   float2* z;
   float* sigma2;
   float* llr;

@@ -34,7 +34,6 @@ namespace {
 
 constexpr int kRefineThreadsMax = 512;   // per system: 2 S threads, 128..512
 constexpr int kFuseThreads = 256;
-constexpr float kCondFp64 = 1e4f;        // condition estimate above which the residual is FP64
 
 // Shared memory of one system (cluster c of subcarrier k; S antennas).  The two
 // U x U scratch areas serve the steps before the last one (the full next
@@ -42,7 +41,7 @@ constexpr float kCondFp64 = 1e4f;        // condition estimate above which the r
 // systems share an SM.
 struct RefineLayout {
   int U, NS, S, SS, W;
-  size_t hs, pm, va, rb, rr, an, ae, cn, total;   // offsets in bytes
+  size_t hs, pm, va, rb, rr, an, ae, total;   // offsets in bytes
   __host__ __device__ RefineLayout(int U_, int NS_, int S_, bool full = true)
       : U(U_), NS(NS_), S(S_), SS(S_ + 1), W(U_ + NS_) {
     size_t o = 0;
@@ -53,8 +52,7 @@ struct RefineLayout {
     rr = o;  o += static_cast<size_t>(NS) * U * 8;      // residual
     an = o;  o += full ? static_cast<size_t>(U) * U * 8 : 0;   // next inverse (FP64 residual: E)
     ae = o;  o += full ? static_cast<size_t>(U) * U * 8 : 0;   // next inverse with the FP64 residual
-    cn = o;  o += static_cast<size_t>(2) * U * 4;       // column norms for the condition estimate
-    total = o;
+    total = o + static_cast<size_t>(2) * U * 4;        // (the plan's limit counts two columns more)
   }
 };
 
@@ -147,38 +145,23 @@ __global__ void __launch_bounds__(kRefineThreadsMax) refine_system_kernel(const 
   const float2* Hk = p.H + static_cast<size_t>(k) * U * B + p.cl_off[c];
   const float2* yk = p.y + static_cast<size_t>(k) * NS * B + p.cl_off[c];
 
+  // Wait for the solve kernel (programmatic dependent launch), then its results.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // Residual precision of this system (block-uniform): the solve kernel marked
+  // the systems whose condition estimate exceeds kCondFp64.
+  const int mark = p.fails[sys];
+  const bool failed = (mark & kRefinePivotMask) != 0;
+  const bool use64 = p.res64 == 2 || (p.res64 == 1 && (mark & kRefineFp64Mark) != 0);
+  if (p.only64 && !use64) return;   // refine_tile_kernel takes it
   for (int e = tid; e < U * S; e += nt) {
     const int u = e / S, b = e - u * S;
     Hs[u * SS + b] = Hk[static_cast<size_t>(u) * B + b];
   }
-  // Wait for the solve kernel (programmatic dependent launch), then its results.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int e = tid; e < W * U; e += nt) {
     const int j = e / U, i = e - j * U;
     P[e] = j < U ? p.As[(sys * U + j) * U + i] : p.Xs[(sys * NS + (j - U)) * U + i];
   }
   __syncthreads();
-  const bool failed = p.fails[sys] != 0;
-  // Residual precision of this system (block-uniform).  Condition estimate:
-  // ||G_c + rho I||_1 from the contraction output (row v of D is column v of the
-  // Hermitian G_c) times ||A~_c||_1.
-  bool use64 = p.res64 == 2;
-  if (p.res64 == 1) {
-    float* cs = reinterpret_cast<float*>(smem + L.cn);
-    for (int j = tid; j < 2 * U; j += nt) {
-      const float2* col = j < U ? p.D + (sys * W + j) * U : P + (j - U) * U;
-      float s = j < U ? rho : 0.f;
-      for (int i = 0; i < U; ++i) s += sqrtf(fmaf(col[i].x, col[i].x, col[i].y * col[i].y));
-      cs[j] = s;
-    }
-    __syncthreads();
-    float mg = 0.f, ma = 0.f;
-    for (int j = 0; j < U; ++j) {
-      mg = fmaxf(mg, cs[j]);
-      ma = fmaxf(ma, cs[U + j]);
-    }
-    use64 = mg * ma > kCondFp64;
-  }
 
   for (int step = 0; step < p.steps && !failed; ++step) {
     if (!use64) {
@@ -328,23 +311,305 @@ __global__ void __launch_bounds__(kRefineThreadsMax) refine_system_kernel(const 
       if (j < U && part == 0) P[j * U + j] = cadd(P[j * U + j], d);
     }
     __syncthreads();
-  }  // Refined estimates and the diagonal of the refined inverse (all that the
-  // fusion kernel reads) back to the workspace, in the same layouts.
+  }
+  // All that the fusion kernel reads back to the workspace: the refined
+  // estimates, and per user the diagonal of the refined inverse with G_uu, packed
+  // at the start of the system's inverse.
   for (int e = tid; e < U + NS * U; e += nt) {
-    if (e < U) p.As[(sys * U + e) * U + e] = P[e * U + e];
+    if (e < U) p.As[sys * U * U + e] = make_float2(P[e * U + e].x, p.D[(sys * W + e) * U + e].x);
     else p.Xs[sys * NS * U + (e - U)] = P[U * U + (e - U)];
   }
   // Let the fusion kernel start its launch while this grid drains.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Warps per system of the tile kernel: 16 antennas each, at most 8.
+inline int refine_tile_warps(int S) { return S <= 16 ? 1 : (S >= 128 ? 8 : (S + 15) / 16); }
+
+// One FP32 refinement step of one system, as register tiles (what a call with one
+// step runs for every system that does not take the FP64 residual).
+//
+// A CTA of NW warps per system.  The generic kernel above computes each product
+// from 2 x 2 tiles (8 bytes of shared memory per complex FMA, where an SM feeds
+// its FMA lanes with 4), which kept the shared-memory pipe 97% busy; here
+//   V = H_c [A~ | X]      tiles of 4 antennas x CPL columns per lane, two users per
+//                         16-byte load: 3.3 bytes per complex FMA,
+//   r = H_c^H (y - H_c x) tiles of NI symbols x JU users, two antennas per load,
+//   x + A~ r              the same tiles,
+// V stays in registers (only its column norms and y - H_c x are kept), and a
+// 16-antenna cluster needs one warp, so that nine systems share an SM.  Measured
+// on 52,800 systems (S = 16, U = 32, 14 symbols): see refine_system_kernel's
+// launch below.  Antennas are padded to 16, users to 2 with zeros.
+template <int UP, int NI>
+struct RefineTile {
+  static constexpr int JU = UP / 8;                        // users per lane (8 user lanes)
+  static constexpr int CPL = (UP + 4 * NI + 7) / 8;        // columns of [A~ | X] per lane
+};
+
+struct RefineTileLayout {
+  int S16, SS, U2, US;                  // padded antennas and users, row strides (complex)
+  size_t hs, pm, rb, rr, vn, total;
+  __host__ __device__ RefineTileLayout(int U, int NS, int S, int NW) {
+    S16 = S < 1 ? 16 : (S + 15) / 16 * 16;
+    SS = S16 + 2;                       // rows 16 bytes apart in the banks
+    U2 = (U + 1) / 2 * 2;
+    US = (U2 + 13) / 16 * 16 + 2;       // the same for the columns of A~ and X
+    if (US < U2) US += 16;
+    size_t o = 0;
+    hs = o;  o += static_cast<size_t>(U2) * SS * 8;
+    pm = o;  o += static_cast<size_t>(U + NS) * US * 8;
+    rb = o;  o += static_cast<size_t>(NS) * SS * 8;
+    rr = o;  o += static_cast<size_t>(NW) * NS * US * 8;   // residual (partial sums per warp)
+    vn = o;  o += static_cast<size_t>(S16 / 16) * U * 4;    // column norms of V per 16 antennas
+    total = (o + 15) / 16 * 16;
+  }
+};
+
+// Asynchronous copy of `rows` rows of `cols` complex values (source stride lds,
+// shared stride ldd, even) by nt threads: 16-byte pieces where the rows allow.
+__device__ __forceinline__ void copy_rows(float2* dst, int ldd, const float2* src, int lds, int rows, int cols, int tid,
+                                          int nt) {
+  if (cols <= 0) return;
+  const int w = ((cols | lds) & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0 ? 2 : 1;   // values per piece
+  const int per = cols / w;
+  int row = tid / per, e = tid - row * per;
+  const int drow = nt / per, de = nt - drow * per;
+  while (row < rows) {
+    const uint32_t d = smem_u32(dst + row * ldd + w * e);
+    const float2* s = src + static_cast<size_t>(row) * lds + w * e;
+    if (w == 2)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(s) : "memory");
+    else
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(s) : "memory");
+    row += drow;
+    e += de;
+    if (e >= per) {
+      e -= per;
+      ++row;
+    }
+  }
+}
+
+template <int UP, int NI>
+__global__ void __launch_bounds__(256, 2) refine_tile_kernel(const RefineParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  using T = RefineTile<UP, NI>;
+  constexpr int JU = T::JU, CPL = T::CPL;
+  const size_t sys = blockIdx.x;
+  const int U = p.U, NS = p.n_sym, Ceff = p.Ceff, B = p.B;
+  const int k = static_cast<int>(sys / Ceff), c = static_cast<int>(sys % Ceff);
+  const int S = p.cl_off[c + 1] - p.cl_off[c];
+  const int tid = threadIdx.x, nt = blockDim.x, NW = nt / 32, warp = tid >> 5, lane = tid & 31;
+  const RefineTileLayout L(U, NS, S, NW);
+  const int SS = L.SS, US = L.US, W = U + NS, S16 = L.S16;
+  float2* Hs = reinterpret_cast<float2*>(smem + L.hs);
+  float2* P = reinterpret_cast<float2*>(smem + L.pm);
+  float2* Rb = reinterpret_cast<float2*>(smem + L.rb);
+  float2* Rr = reinterpret_cast<float2*>(smem + L.rr);
+  float* vn = reinterpret_cast<float*>(smem + L.vn);
+  const float rho = p.rho;
+  // H_c and y_c with zero antennas up to S16 and a zero user up to U2.
+  const float2* Hk = p.H + static_cast<size_t>(k) * U * B + p.cl_off[c];
+  const float2* yk = p.y + static_cast<size_t>(k) * NS * B + p.cl_off[c];
+  copy_rows(Hs, SS, Hk, B, U, S, tid, nt);
+  copy_rows(Rb, SS, yk, B, NS, S, tid, nt);
+  if (S16 != S) {
+    const int pad = S16 - S;
+    for (int e = tid; e < (U + NS) * pad; e += nt) {
+      const int row = e / pad, b = S + e - row * pad;
+      (row < U ? Hs + row * SS : Rb + (row - U) * SS)[b] = make_float2(0.f, 0.f);
+    }
+  }
+  if (L.U2 != U)
+    for (int b = tid; b < S16; b += nt) Hs[U * SS + b] = make_float2(0.f, 0.f);
+  // Wait for the solve kernel (programmatic dependent launch), then its results.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int mark = p.fails[sys];
+  if (p.res64 == 1 && (mark & kRefineFp64Mark)) {   // the generic kernel takes it
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return;
+  }
+  copy_rows(P, US, p.As + sys * U * U, U, U, U, tid, nt);
+  copy_rows(P + U * US, US, p.Xs + sys * NS * U, U, NS, U, tid, nt);
+  if (L.U2 != U)
+    for (int j = tid; j < W; j += nt) P[j * US + U] = make_float2(0.f, 0.f);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  const bool failed = (mark & kRefinePivotMask) != 0;
+
+  // V = H_c [A~ | X]: lane (r, q) has antennas 16 ta + 4 r .. + 3 and columns q + 8 j.
+  if (!failed) {
+    const int r = lane >> 3, q = lane & 7;
+    const float2* pc[CPL];
+#pragma unroll
+    for (int j = 0; j < CPL; ++j) pc[j] = P + (q + 8 * j < W ? q + 8 * j : 0) * US;
+    for (int ta = warp; ta < S16 / 16; ta += NW) {
+      const float2* hp = Hs + 16 * ta + 4 * r;
+      float2 acc[4][CPL];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < CPL; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      for (int u = 0; u < U; u += 2) {
+        float4 h0[2], h1[2];   // users u and u + 1, four antennas each
+        h0[0] = *reinterpret_cast<const float4*>(hp + u * SS);
+        h0[1] = *reinterpret_cast<const float4*>(hp + u * SS + 2);
+        h1[0] = *reinterpret_cast<const float4*>(hp + (u + 1) * SS);
+        h1[1] = *reinterpret_cast<const float4*>(hp + (u + 1) * SS + 2);
+#pragma unroll
+        for (int j = 0; j < CPL; ++j) {
+          const float4 a = *reinterpret_cast<const float4*>(pc[j] + u);
+          const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            acc[2 * h][j] = cfma(make_float2(h0[h].x, h0[h].y), a0, acc[2 * h][j]);
+            acc[2 * h][j] = cfma(make_float2(h1[h].x, h1[h].y), a1, acc[2 * h][j]);
+            acc[2 * h + 1][j] = cfma(make_float2(h0[h].z, h0[h].w), a0, acc[2 * h + 1][j]);
+            acc[2 * h + 1][j] = cfma(make_float2(h1[h].z, h1[h].w), a1, acc[2 * h + 1][j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < CPL; ++j) {
+        const int col = q + 8 * j;
+        // Columns of A~: their norm; columns of X: y - H_c x in place of y.
+        float s = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s += cabs2(acc[i][j]);
+        s += __shfl_xor_sync(kFullMask, s, 8);
+        s += __shfl_xor_sync(kFullMask, s, 16);
+        if (col < U) {
+          if (r == 0) vn[ta * U + col] = s;
+        } else if (col < W) {
+          float2* at = Rb + (col - U) * SS + 16 * ta + 4 * r;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) at[i] = csub(at[i], acc[i][j]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // r = H_c^H (y_c - H_c x): lane (r, q) has symbols r + 4 i and users q + 8 j; the
+  // antennas are split over the warps (whole pairs).
+  if (!failed) {
+    const int r = lane >> 3, q = lane & 7;
+    const int pairs = S16 / 2, p0 = pairs * warp / NW, p1 = pairs * (warp + 1) / NW;
+    const float2* hu[JU];
+    const float2* rn[NI];
+#pragma unroll
+    for (int j = 0; j < JU; ++j) hu[j] = Hs + (q + 8 * j < U ? q + 8 * j : 0) * SS;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) rn[i] = Rb + (r + 4 * i < NS ? r + 4 * i : 0) * SS;
+    float2 acc[NI][JU];
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < JU; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    for (int b = 2 * p0; b < 2 * p1; b += 2) {
+      float4 h[JU];
+#pragma unroll
+      for (int j = 0; j < JU; ++j) h[j] = *reinterpret_cast<const float4*>(hu[j] + b);
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const float4 y = *reinterpret_cast<const float4*>(rn[i] + b);
+#pragma unroll
+        for (int j = 0; j < JU; ++j) {
+          acc[i][j] = cfma_conj(make_float2(h[j].x, h[j].y), make_float2(y.x, y.y), acc[i][j]);
+          acc[i][j] = cfma_conj(make_float2(h[j].z, h[j].w), make_float2(y.z, y.w), acc[i][j]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < JU; ++j) {
+        const int n = r + 4 * i, u = q + 8 * j;
+        if (n < NS && u < U) Rr[(warp * NS + n) * US + u] = acc[i][j];
+      }
+  }
+  __syncthreads();
+  if (!failed) {
+    // The parts in warp order, minus rho x.
+    for (int e = tid; e < NS * U; e += nt) {
+      const int n = e / U, u = e - n * U;
+      float2 v = Rr[n * US + u];
+      for (int w = 1; w < NW; ++w) v = cadd(v, Rr[(w * NS + n) * US + u]);
+      const float2 x = P[(U + n) * US + u];
+      Rr[n * US + u] = make_float2(v.x - rho * x.x, v.y - rho * x.y);
+    }
+  }
+  __syncthreads();
+  // x + A~ r to the workspace: lane (r, q) has users JU q .. and symbols r + 4 i, the
+  // symbol rows i split over the warps.
+  {
+    const int r = lane >> 3, q = lane & 7;
+    for (int i0 = warp; i0 < NI; i0 += NW) {
+      const int rows = NW == 1 ? NI : 1;
+      float2 acc[NI][JU];
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int j = 0; j < JU; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      const int ub = JU * q < U ? JU * q : 0;
+      if (!failed) {
+        for (int v = 0; v < U; ++v) {
+          float2 a[JU];
+#pragma unroll
+          for (int j = 0; j < JU; ++j) a[j] = P[v * US + ub + j];
+#pragma unroll
+          for (int i = 0; i < NI; ++i) {
+            if (i < rows) {
+              const int n = r + 4 * (i0 + i);
+              const float2 rv = Rr[(n < NS ? n : 0) * US + v];
+#pragma unroll
+              for (int j = 0; j < JU; ++j) acc[i][j] = cfma(a[j], rv, acc[i][j]);
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        if (i < rows) {
+          const int n = r + 4 * (i0 + i);
+#pragma unroll
+          for (int j = 0; j < JU; ++j) {
+            const int u = JU * q + j;
+            if (n < NS && u < U) p.Xs[(sys * NS + n) * U + u] = cadd(P[(U + n) * US + u], acc[i][j]);
+          }
+        }
+      }
+      if (NW == 1) break;
+    }
+  }
+  // [2 A - V^H V - rho A^H A]_jj per user (the part of the next inverse that is
+  // read), packed with G_jj at the start of the system's inverse.
+  for (int j = tid; j < U; j += nt) {
+    float d = P[j * US + j].x;
+    if (!failed) {
+      float d1 = 0.f, d2 = 0.f;
+      for (int ta = 0; ta < S16 / 16; ++ta) d1 += vn[ta * U + j];
+      for (int v = 0; v < U; ++v) {
+        const float2 a = P[j * US + v];
+        d2 = fmaf(a.x, a.x, fmaf(a.y, a.y, d2));
+      }
+      d = fmaf(-rho, d2, 2.f * d - d1);
+    }
+    p.As[sys * U * U + j] = make_float2(d, p.D[(sys * W + j) * U + j].x);
+  }
+  // Let the next kernel start its launch while this grid drains.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Per subcarrier: fusion terms from the refined systems (as the solve kernel:
-// weight g / A_uu with g = mu or 1), sum over clusters, z, sigma^2 and LLRs.
+// weight g / A_uu with g = mu or 1), sum over clusters, z, sigma^2 and LLRs.  The
+// estimates are read straight from the workspace, coalesced over the users, one
+// output per thread (staging all of them in shared memory first left 3 CTAs per
+// SM).
 __global__ void __launch_bounds__(kFuseThreads) refine_fuse_kernel(const RefineParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int U = p.U, NS = p.n_sym, Ceff = p.Ceff, W = U + NS;
-  float2* Fz = reinterpret_cast<float2*>(smem);                        // [Ceff][NS][U]
-  float* Dn = reinterpret_cast<float*>(Fz + static_cast<size_t>(Ceff) * NS * U);   // [Ceff][U]
+  const int U = p.U, NS = p.n_sym, Ceff = p.Ceff;
+  float* Ia = reinterpret_cast<float*>(smem);                          // [Ceff][U]: 1 / A_uu
+  float* Dn = Ia + static_cast<size_t>(Ceff) * U;                      // [Ceff][U]
   int* failed = reinterpret_cast<int*>(Dn + static_cast<size_t>(Ceff) * U);
   const int k = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const size_t sys0 = static_cast<size_t>(k) * Ceff;
@@ -352,16 +617,14 @@ __global__ void __launch_bounds__(kFuseThreads) refine_fuse_kernel(const RefineP
   if (tid == 0) *failed = 0;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();
-  if (tid < Ceff && p.fails[sys0 + tid] != 0) atomicOr(failed, 1);
+  if (tid < Ceff && (p.fails[sys0 + tid] & kRefinePivotMask) != 0) atomicOr(failed, 1);
   for (int e = tid; e < Ceff * U; e += nt) {
     const int c = e / U, u = e - c * U;
-    const size_t sys = sys0 + c;
-    const float gii = p.D[(sys * W + u) * U + u].x;
-    const float A = p.As[(sys * U + u) * U + u].x;
-    const float invA = 1.f / A;
-    const float mu = gii == 0.f ? 0.f : fmaxf(1.f - rho * A, 0.f);
+    const float2 ag = p.As[(sys0 + c) * U * U + u];   // A_uu, G_uu
+    const float invA = 1.f / ag.x;
+    const float mu = ag.y == 0.f ? 0.f : fmaxf(1.f - rho * ag.x, 0.f);
+    Ia[e] = invA;
     Dn[e] = (p.unbiased ? mu : 1.f) * invA;
-    for (int n = 0; n < NS; ++n) Fz[(c * NS + n) * U + u] = cscale(p.Xs[(sys * NS + n) * U + u], invA);
   }
   __syncthreads();
   const int bits = p.llr_bits, hb = bits / 2;
@@ -370,8 +633,9 @@ __global__ void __launch_bounds__(kFuseThreads) refine_fuse_kernel(const RefineP
     const int n = e / U, u = e - n * U;
     float2 nm = make_float2(0.f, 0.f);
     float dn = 0.f;
+#pragma unroll 4
     for (int c = 0; c < Ceff; ++c) {
-      nm = cadd(nm, Fz[(c * NS + n) * U + u]);
+      nm = cadd(nm, cscale(p.Xs[(sys0 + c) * NS * U + e], Ia[c * U + u]));
       dn += Dn[c * U + u];
     }
     float2 zz;
@@ -390,7 +654,7 @@ __global__ void __launch_bounds__(kFuseThreads) refine_fuse_kernel(const RefineP
     const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
     p.z[zi] = zz;
     if (n == 0) p.sigma2[static_cast<size_t>(k) * U + u] = s2;
-    if (bits) symbol_llr(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
+    if (bits) symbol_llr_wide(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
   }
 }
 
@@ -416,7 +680,37 @@ bool refine_fits(int max_S, int U, int n_sym) { return RefineLayout(U, n_sym, ma
 
 size_t refine_smem_bytes(int max_S, int U, int n_sym) { return RefineLayout(U, n_sym, max_S).total; }
 
-cudaError_t launch_refine(const RefineParams& p, cudaStream_t stream) {
+namespace {
+
+template <int UP, int NI>
+cudaError_t launch_tile(const RefineParams& p, cudaStream_t stream) {
+  static int configured[64] = {0};
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if (dev < 64 && !configured[dev]) {
+    err = cudaFuncSetAttribute(refine_tile_kernel<UP, NI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (err != cudaSuccess) return err;
+    configured[dev] = 1;
+  }
+  const int NW = refine_tile_warps(p.max_S);
+  return launch_pdl(reinterpret_cast<const void*>(refine_tile_kernel<UP, NI>),
+                    dim3(static_cast<unsigned>(static_cast<size_t>(p.n_sc) * p.Ceff)), dim3(32 * NW),
+                    RefineTileLayout(p.U, p.n_sym, p.max_S, NW).total, stream, p);
+}
+
+cudaError_t launch_tile_any(const RefineParams& p, cudaStream_t stream) {
+  const bool wide = p.n_sym > 4;
+  switch (padded_users(p.U)) {
+    case 8: return wide ? launch_tile<8, 4>(p, stream) : launch_tile<8, 1>(p, stream);
+    case 16: return wide ? launch_tile<16, 4>(p, stream) : launch_tile<16, 1>(p, stream);
+    default: return wide ? launch_tile<32, 4>(p, stream) : launch_tile<32, 1>(p, stream);
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_refine(const RefineParams& base, cudaStream_t stream) {
   static int configured[64] = {0};
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
@@ -428,13 +722,25 @@ cudaError_t launch_refine(const RefineParams& p, cudaStream_t stream) {
     if (err != cudaSuccess) return err;
     configured[dev] = 1;
   }
+  RefineParams p = base;
   const size_t nsys = static_cast<size_t>(p.n_sc) * p.Ceff;
   const int S = p.max_S;   // shared memory and threads for the largest cluster
-  const int threads = 2 * S < 128 ? 128 : (2 * S > kRefineThreadsMax ? kRefineThreadsMax : ((2 * S + 31) / 32) * 32);
-  err = launch_pdl(reinterpret_cast<const void*>(refine_system_kernel), dim3(static_cast<unsigned>(nsys)),
-                   dim3(threads), RefineLayout(p.U, p.n_sym, S, p.steps > 1).total, stream, p);
-  if (err != cudaSuccess) return err;
-  const size_t fsmem = static_cast<size_t>(p.Ceff) * p.n_sym * p.U * 8 + static_cast<size_t>(p.Ceff) * p.U * 4 + 16;
+  // One FP32 step (of every system, or of those below the condition threshold):
+  // the tile kernel, where its padded layout fits.
+  const bool tiles = p.steps == 1 && p.res64 != 2 &&
+                     RefineTileLayout(p.U, p.n_sym, S, refine_tile_warps(S)).total <= 227 * 1024;
+  if (tiles) {
+    err = launch_tile_any(p, stream);
+    if (err != cudaSuccess) return err;
+  }
+  p.only64 = tiles ? 1 : 0;
+  if (!tiles || p.res64 == 1) {
+    const int threads = 2 * S < 128 ? 128 : (2 * S > kRefineThreadsMax ? kRefineThreadsMax : ((2 * S + 31) / 32) * 32);
+    err = launch_pdl(reinterpret_cast<const void*>(refine_system_kernel), dim3(static_cast<unsigned>(nsys)),
+                     dim3(threads), RefineLayout(p.U, p.n_sym, S, p.steps > 1).total, stream, p);
+    if (err != cudaSuccess) return err;
+  }
+  const size_t fsmem = static_cast<size_t>(p.Ceff) * p.U * 8 + 16;
   return launch_pdl(reinterpret_cast<const void*>(refine_fuse_kernel), dim3(p.n_sc), dim3(kFuseThreads), fsmem,
                     stream, p);
 }

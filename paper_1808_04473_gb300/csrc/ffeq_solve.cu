@@ -233,12 +233,14 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? (UP <= 16 ? 5 : 3) : 1) so
     const bool live = m < nmat && sc < p.n_sc;
     const size_t sys = static_cast<size_t>(live ? sc : 0) * Ceff + (live ? c : 0);
     float2* Fz = areas + static_cast<size_t>(m < nmat ? m : 0) * Lay::kArea;
-    const int fail = tile_solve_system<UP, NRC>(p.D + sys * mat, U, NS, p.rho, p.unbiased, live, lane_ok && m < nmat, r, q,
-                                           buf, Fz, reinterpret_cast<float*>(Fz + kNsymMax * UP),
-                                           p.Xs ? p.Xs + sys * NS * U : nullptr, p.Xs ? p.As + sys * U * U : nullptr);
+    float cond = 0.f;
+    const int fail = tile_solve_system<UP, NRC>(
+        p.D + sys * mat, U, NS, p.rho, p.unbiased, live, lane_ok && m < nmat, r, q, buf, Fz,
+        reinterpret_cast<float*>(Fz + kNsymMax * UP), p.Xs ? p.Xs + sys * NS * U : nullptr,
+        p.Xs ? p.As + sys * U * U : nullptr, cond);
     if (gl == 0 && live) {
       if (p.info) p.info[sys] = fail;
-      if (p.Xs) p.fails[sys] = fail;
+      if (p.Xs) p.fails[sys] = fail | (p.cond && cond > kCondFp64 ? kRefineFp64Mark : 0);
       else if (fail) atomicOr(&fail_sc[scl], 1);
     }
   }
@@ -550,7 +552,10 @@ cudaError_t launch_batch_up(const SolveParams& p, cudaStream_t stream) {
 // throughput workload's 1200 CTAs in 1.6 waves) ran faster than a cap of 64
 // with spills and one wave (FD 24.7 -> 23.1 us alone, and the concurrent
 // PD + FD step 75.2 -> 70.7 us).
-template <int UP>
+// COND: refinement follows and wants the condition estimate in the status word (a
+// kernel of its own: it costs the plain one 3%, 697 -> 720 us for U = 32, C = 16,
+// 3300 x 14).
+template <int UP, bool COND>
 __global__ void __launch_bounds__(512, 1) solve_full_kernel(const SolveParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Lay = SolveLayout<UP>;
@@ -595,6 +600,11 @@ __global__ void __launch_bounds__(512, 1) solve_full_kernel(const SolveParams p)
   // Lane i: row i of A = (G + rho I)^{-1} (natural column order) and A_ii.
   float2 arow[UP];
   float Ai, gii;
+  float gnorm = rho;                    // row i of ||G_c + rho I||_1 (G_c is Hermitian)
+  if constexpr (COND) {
+#pragma unroll
+    for (int j = 0; j < UP; ++j) gnorm += sqrt_approx(cabs2(mrow[j]));
+  }
   const int fail = gj_solve_row<UP>(mrow, rho, reinterpret_cast<float*>(rowbuf), i, g < nmat, arow, Ai, gii);
   const float invA = rcp_approx(Ai);
   // mu = [A G]_ii = 1 - rho A_ii; a user the cluster cannot see (G_ii = 0) has
@@ -629,12 +639,24 @@ __global__ void __launch_bounds__(512, 1) solve_full_kernel(const SolveParams p)
     }
   }
   if (store) {
+    int mark = 0;
+    if constexpr (COND) {
+      float anorm = 0.f;
+#pragma unroll
+      for (int j = 0; j < UP; ++j) anorm += sqrt_approx(fmaf(are[j].x, are[j].x, aim[j].x * aim[j].x));
+#pragma unroll
+      for (int o = UP / 2; o > 0; o >>= 1) {
+        gnorm = fmaxf(gnorm, __shfl_xor_sync(kFullMask, gnorm, o));
+        anorm = fmaxf(anorm, __shfl_xor_sync(kFullMask, anorm, o));
+      }
+      if (gnorm * anorm > kCondFp64) mark = kRefineFp64Mark;
+    }
     // Inverse stored transposed (row j = column j of A, coalesced over the lanes i).
     if (live) {
 #pragma unroll
       for (int j = 0; j < UP; ++j) p.As[(sys * U + j) * U + i] = make_float2(are[j].x, aim[j].x);
       if (i == 0) {
-        p.fails[sys] = fail;
+        p.fails[sys] = fail | mark;
         if (p.info) p.info[sys] = fail;
       }
     }
@@ -684,8 +706,8 @@ __global__ void __launch_bounds__(512, 1) solve_full_kernel(const SolveParams p)
   }
 }
 
-template <int UP>
-cudaError_t launch_full(const SolveParams& p, cudaStream_t stream) {
+template <int UP, bool COND>
+cudaError_t launch_full_as(const SolveParams& p, cudaStream_t stream) {
   using Lay = SolveLayout<UP>;
   const int nmat = p.spc * p.Ceff;
   const int threads = ((nmat * UP + 31) / 32) * 32;
@@ -695,7 +717,7 @@ cudaError_t launch_full(const SolveParams& p, cudaStream_t stream) {
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   if (dev < 64 && !configured[dev]) {
-    err = cudaFuncSetAttribute(solve_full_kernel<UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    err = cudaFuncSetAttribute(solve_full_kernel<UP, COND>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (err != cudaSuccess) return err;
     configured[dev] = 1;
   }
@@ -709,7 +731,12 @@ cudaError_t launch_full(const SolveParams& p, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, solve_full_kernel<UP>, p);
+  return cudaLaunchKernelEx(&cfg, solve_full_kernel<UP, COND>, p);
+}
+
+template <int UP>
+cudaError_t launch_full(const SolveParams& p, cudaStream_t stream) {
+  return p.cond ? launch_full_as<UP, true>(p, stream) : launch_full_as<UP, false>(p, stream);
 }
 
 // Maximum-ratio combining (Sec. III-A) per (subcarrier, cluster), uniform

@@ -125,12 +125,14 @@ __device__ __forceinline__ int tile_sweep(float (&re)[4][UP / 4 + NRC], float (&
 // denominators g_{c,u} / A_uu (g = mu or 1) in Dn; or (Xs != nullptr: refinement
 // follows) writes the estimates Xs [n][U] and the inverse As [j][i] = A[i][j] to
 // global memory.  A group without a system (valid = false) sweeps an identity;
-// nothing is left where `writer` is false.  Every lane of the warp takes part;
+// nothing is left where `writer` is false, and cond is the condition estimate
+// ||G + rho I||_1 ||A||_1.  Every lane of the warp takes part;
 // returns the sweep's failure index.
 template <int UP, int NRC>
 __device__ __forceinline__ int tile_solve_system(const float2* __restrict__ Dg, int U, int NS, float rho, bool unbiased,
                                                  bool valid, bool writer, int r, int q, float* buf,
-                                                 float2* Fz, float* Dn, float2* Xs, float2* As) {
+                                                 float2* Fz, float* Dn, float2* Xs, float2* As,
+                                                 float& cond) {
   constexpr int CA = UP / 4, NC = CA + NRC;
   float re[4][NC], im[4][NC];
   const int row0 = 4 * r;
@@ -178,9 +180,30 @@ __device__ __forceinline__ int tile_solve_system(const float2* __restrict__ Dg, 
       }
     }
   }
-  float rs[4];
+  constexpr int GL = TileShape<UP, NRC>::GL;
+  // max over the group of the rows' absolute sums (rows scaled by s): the 1-norm
+  // of a Hermitian matrix.
+  auto norm1 = [&](const float (&s)[4]) {
+    float most = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < CA; ++j)
+        if (CA * q + j < U && row0 + i < U) sum += sqrt_approx(fmaf(re[i][j], re[i][j], im[i][j] * im[i][j]));
+      sum += __shfl_xor_sync(kFullMask, sum, 1);
+      sum += __shfl_xor_sync(kFullMask, sum, 2);
+      most = fmaxf(most, sum * fabsf(s[i]));
+    }
+#pragma unroll
+    for (int o = GL / 2; o >= 4; o >>= 1) most = fmaxf(most, __shfl_xor_sync(kFullMask, most, o));
+    return most;
+  };
+  float rs[4] = {1.f, 1.f, 1.f, 1.f};
+  if (Xs) cond = norm1(rs);
   const int fail = tile_sweep<UP, NRC>(re, im, r, q, rs);
   if (Xs) {
+    cond *= norm1(rs);
     if (valid && writer) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
