@@ -40,7 +40,11 @@ namespace {
 // Gaussian noise of variance tau/2 per axis:
 // p(a_m | x) ~ exp(-(x - a_m)^2 / tau) = 2^(-(x - a_m)^2 log2(e) / tau).
 // Exponents are taken relative to the nearest level a0, and the moments about
-// a0, so that a sharp posterior on an outer level keeps its small variance.
+// a0, so that a sharp posterior on an outer level keeps its small variance: with
+// e = a_m - a0 and r0 = x - a0, (x - a0)^2 - (x - a_m)^2 = e (2 r0 - e).  The
+// nearest level itself weighs 1 and adds nothing to the moments, so only the
+// other L - 1 are visited, in the order m0 + 1, m0 + 2, ... modulo L (e is then
+// one of two constants per visit).
 // The two axes run as the halves of paired FP32 operations (__ffma2_rn and
 // friends, sm_100+), each half rounding as the scalar operation would.
 // inv_d = 1/d; l2t = log2(e) / tau (both once per call site, not per level).
@@ -54,20 +58,20 @@ __device__ __forceinline__ void pam_posterior2(float2 x, float l2t, float d, flo
   const float2 a0 = __fmul2_rn(__ffma2_rn(q, make_float2(2.f, 2.f), make_float2(1.f - L, 1.f - L)),
                                make_float2(d, d));
   const float2 r0 = __ffma2_rn(a0, make_float2(-1.f, -1.f), x);          // x - a0
-  const float2 ne0 = __fmul2_rn(r0, make_float2(-r0.x, -r0.y));           // -(x - a0)^2
   const float2 nl2t = make_float2(-l2t, -l2t);
-  const float2 na0 = make_float2(-a0.x, -a0.y);
-  float2 sw = make_float2(0.f, 0.f), s1 = sw, s2 = sw;
+  const float2 rl = __fmul2_rn(r0, make_float2(2.f * l2t, 2.f * l2t));   // 2 r0 l2t
+  float2 sw = make_float2(1.f, 1.f), s1 = make_float2(0.f, 0.f), s2 = s1;
 #pragma unroll
-  for (int m = 0; m < L; ++m) {
-    const float a = (2.f * static_cast<float>(m) - static_cast<float>(L - 1)) * d;
-    const float2 e = __fadd2_rn(x, make_float2(-a, -a));                  // x - a
-    const float2 u = __fmul2_rn(__ffma2_rn(e, e, ne0), nl2t);             // ((x-a0)^2 - e^2) l2t <= 0
-    const float2 w = make_float2(ex2_approx(u.x), ex2_approx(u.y));       // 1 at a0
-    const float2 da = __fadd2_rn(make_float2(a, a), na0);
+  for (int m = 1; m < L; ++m) {
+    const float up = 2.f * static_cast<float>(m) * d, down = 2.f * static_cast<float>(m - L) * d;
+    const float wrap = static_cast<float>(L - m);                         // m0 + m >= L: the level m - L steps away
+    const float2 e = make_float2(q.x >= wrap ? down : up, q.y >= wrap ? down : up);   // a_m - a0
+    const float2 u = __fmul2_rn(e, __ffma2_rn(e, nl2t, rl));              // ((x-a0)^2 - (x-a_m)^2) l2t <= 0
+    const float2 w = make_float2(ex2_approx(u.x), ex2_approx(u.y));
+    const float2 we = __fmul2_rn(w, e);
     sw = __fadd2_rn(sw, w);
-    s1 = __ffma2_rn(w, da, s1);
-    s2 = __ffma2_rn(__fmul2_rn(w, da), da, s2);
+    s1 = __fadd2_rn(s1, we);
+    s2 = __ffma2_rn(we, e, s2);
   }
   const float2 r = make_float2(rcp_approx(sw.x), rcp_approx(sw.y));   // sw >= 1
   const float2 m1 = __fmul2_rn(s1, r);
@@ -145,29 +149,32 @@ __device__ __forceinline__ void lama_block(const LamaUnit& w, unsigned char* sme
     // iteration's stores before the loads, and the buffer written next iteration
     // is the other one (the one after that is only written once every lane has
     // passed the next __syncwarp, i.e. finished these loads).
-    float* cur = (t & 1) ? sb1 : sb0;
-    cur[i] = s.x;
-    cur[UP + i] = s.y;
-    __syncwarp();
-    // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
-    // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
-    float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
+    z = yv;                 // t = 1: s = v = 0
+    if (t > 1) {
+      float* cur = (t & 1) ? sb1 : sb0;
+      cur[i] = s.x;
+      cur[UP + i] = s.y;
+      __syncwarp();
+      // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
+      // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
+      float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
 #pragma unroll
-    for (int j = 0; j < UP; j += 4) {
-      const float4 sr = *reinterpret_cast<const float4*>(cur + j);
-      const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
+      for (int j = 0; j < UP; j += 4) {
+        const float4 sr = *reinterpret_cast<const float4*>(cur + j);
+        const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
-        const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
-        rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
-        ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
-        ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
-        ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
+        for (int h = 0; h < 2; ++h) {
+          const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
+          const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
+          rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
+          ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
+          ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
+          ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
+        }
       }
+      const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
+      z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
     }
-    const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
-    z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
     tau = fmaf(beta, phi, n0n);
     if (t >= w.iters) break;
     const float inv_tau = rcp_approx(tau);
@@ -276,29 +283,32 @@ __global__ void __maxnreg__(UP == 32 ? 128 : 64) lama_kernel(const SolveParams p
     // iteration's stores before the loads, and the buffer written next iteration
     // is the other one (the one after that is only written once every lane has
     // passed the next __syncwarp, i.e. finished these loads).
-    float* cur = (t & 1) ? sb1 : sb0;
-    cur[i] = s.x;
-    cur[UP + i] = s.y;
-    __syncwarp();
-    // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
-    // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
-    float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
+    z = yv;                 // t = 1: s = v = 0
+    if (t > 1) {
+      float* cur = (t & 1) ? sb1 : sb0;
+      cur[i] = s.x;
+      cur[UP + i] = s.y;
+      __syncwarp();
+      // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
+      // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
+      float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
 #pragma unroll
-    for (int j = 0; j < UP; j += 4) {
-      const float4 sr = *reinterpret_cast<const float4*>(cur + j);
-      const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
+      for (int j = 0; j < UP; j += 4) {
+        const float4 sr = *reinterpret_cast<const float4*>(cur + j);
+        const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
-        const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
-        rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
-        ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
-        ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
-        ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
+        for (int h = 0; h < 2; ++h) {
+          const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
+          const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
+          rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
+          ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
+          ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
+          ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
+        }
       }
+      const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
+      z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
     }
-    const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
-    z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
     tau = fmaf(beta, phi, n0n);
     if (t >= p.lama_iters) break;
     const float inv_tau = rcp_approx(tau);
