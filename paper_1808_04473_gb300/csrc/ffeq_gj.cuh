@@ -71,6 +71,22 @@ __device__ __forceinline__ float2 gj_update(float2 g, float2 q, float2 base) {
   return base;
 }
 
+// Rotate the column pairs left once per two padding pivots (pads of them).
+template <int W>
+__device__ __forceinline__ void gj_rotate_padding(float2 (&rp)[W / 2], float2 (&ip)[W / 2], int pads) {
+#pragma unroll 1
+  for (; pads > 0; pads -= 2) {
+    const float2 r0 = rp[0], i0 = ip[0];
+#pragma unroll
+    for (int m = 0; m + 1 < W / 2; ++m) {
+      rp[m] = rp[m + 1];
+      ip[m] = ip[m + 1];
+    }
+    rp[W / 2 - 1] = r0;
+    ip[W / 2 - 1] = i0;
+  }
+}
+
 // Gauss-Jordan sweep with deferred row scaling and paired FMAs.
 //
 // Same system and result layout as gj_sweep_rotating, held as pairs of
@@ -89,17 +105,19 @@ __device__ __forceinline__ float2 gj_update(float2 g, float2 q, float2 base) {
 // (pivot columns 0 and 1: pair 0), each with its own broadcast buffer (one warp
 // barrier per step), followed by a rotation by one pair keep register indices
 // compile-time constants.  rowbuf: 2 (2W + 4) floats, 16-byte aligned.  Returns
-// the 1-based index of the first non-positive pivot, or 0.
+// the 1-based index of the first non-positive pivot, or 0.  `steps` (even, the same
+// for the warp): pivots from there on are padding (identity rows and columns, which
+// change nothing) and only their rotations are made.
 template <int UP, int W>
 __device__ __forceinline__ int gj_sweep_pairs(float2 (&rp)[W / 2], float2 (&ip)[W / 2], float* rowbuf, int i,
-                                              bool writer, float& scale) {
+                                              bool writer, float& scale, int steps = UP) {
   static_assert(W % 4 == 0 && UP % 2 == 0, "paired sweep needs W % 4 == 0 and even UP");
   constexpr int NP = W / 2;                // column pairs
   constexpr int kBuf = 2 * W + 4;          // re plane, im plane, pivot (padded to 16 bytes)
   int fail = 0;
   float my_r = 1.f;
 #pragma unroll 1
-  for (int k = 0; k < UP; k += 2) {
+  for (int k = 0; k < steps; k += 2) {
     static_for<2>([&](auto sc) {
       constexpr int s = decltype(sc)::value;   // pivot column of this step (half s of pair 0)
       float* buf = rowbuf + s * kBuf;
@@ -165,6 +183,7 @@ __device__ __forceinline__ int gj_sweep_pairs(float2 (&rp)[W / 2], float2 (&ip)[
       }
     });
   }
+  gj_rotate_padding<W>(rp, ip, UP - steps);
   __syncwarp();   // the buffers may be reused after the sweep
   scale = my_r;
   return fail;
@@ -193,17 +212,17 @@ __device__ __forceinline__ float2 gj_cmul(float2 a, float2 b) {
 // multiplied by their pivot; the caller scales by the returned 1/p_i).  One warp
 // barrier per two pivots instead of two (two broadcast areas, alternating), and
 // both pivot rows are stored by one instruction.  UP must be even.  rowbuf:
-// 2 (4 W + 16) floats, 16-byte aligned.
+// 2 (4 W + 16) floats, 16-byte aligned.  `steps` as in gj_sweep_pairs.
 template <int UP, int W>
 __device__ __forceinline__ int gj_sweep_block2(float2 (&rp)[W / 2], float2 (&ip)[W / 2], float* rowbuf, int i,
-                                               bool writer, float& scale) {
+                                               bool writer, float& scale, int steps = UP) {
   static_assert(W % 4 == 0 && UP % 2 == 0, "block sweep needs W % 4 == 0 and even UP");
   constexpr int NP = W / 2;                // column pairs
   constexpr int kArea = 4 * W + 16;        // one broadcast area
   int fail = 0;
   float my_r = 1.f;
 #pragma unroll 1
-  for (int k = 0; k < UP; k += 2) {
+  for (int k = 0; k < steps; k += 2) {
     float* area = rowbuf + ((k >> 1) & 1) * kArea;
     float* qk = area;                        // [re plane W][im plane W] of row k
     float* qk1 = area + 2 * W;               // the same for row k + 1
@@ -299,6 +318,7 @@ __device__ __forceinline__ int gj_sweep_block2(float2 (&rp)[W / 2], float2 (&ip)
       ip[m] = ni[m];
     }
   }
+  gj_rotate_padding<W>(rp, ip, UP - steps);
   __syncwarp();   // the areas may be reused after the sweep
   scale = my_r;
   return fail;

@@ -390,13 +390,15 @@ __global__ void __launch_bounds__(512, 1) solve_batch_kernel(const SolveParams p
       rp[m] = make_float2(mrow[2 * m].x, mrow[2 * m + 1].x);
       ip[m] = make_float2(mrow[2 * m].y, mrow[2 * m + 1].y);
     }
+    // Pivots up to the widest system of the warp; the rest is padding.
+    const int steps = (__reduce_max_sync(kFullMask, valid ? U : 1) + 1) & ~1;
     float rs = 1.f;
     // 32 pivots: fuse pivot pairs (half the broadcast rounds); up to 16: the
     // sequential paired sweep is faster (measured).
     if constexpr (UP >= 32) {
-      fail = gj_sweep_block2<UP, UP>(rp, ip, reinterpret_cast<float*>(rowbuf), i, g < nmat, rs);
+      fail = gj_sweep_block2<UP, UP>(rp, ip, reinterpret_cast<float*>(rowbuf), i, g < nmat, rs, steps);
     } else {
-      fail = gj_sweep_pairs<UP, UP>(rp, ip, reinterpret_cast<float*>(rowbuf), i, g < nmat, rs);
+      fail = gj_sweep_pairs<UP, UP>(rp, ip, reinterpret_cast<float*>(rowbuf), i, g < nmat, rs, steps);
     }
     float2 arow[UP];
     float Ai = 1.f;
@@ -417,10 +419,15 @@ __global__ void __launch_bounds__(512, 1) solve_batch_kernel(const SolveParams p
       float2 zn = make_float2(0.f, 0.f);
       if (n < NS) {
 #pragma unroll
-        for (int j = 0; j < UP; j += 2) {
-          const float4 y2 = *reinterpret_cast<const float4*>(ys + n * UP + j);
-          zn = cfma(arow[j], make_float2(y2.x, y2.y), zn);
-          zn = cfma(arow[j + 1], make_float2(y2.z, y2.w), zn);
+        for (int j4 = 0; j4 < UP; j4 += 4) {
+          if (j4 < steps) {   // (users past it: zero)
+#pragma unroll
+            for (int j = j4; j < j4 + 4; j += 2) {
+              const float4 y2 = *reinterpret_cast<const float4*>(ys + n * UP + j);
+              zn = cfma(arow[j], make_float2(y2.x, y2.y), zn);
+              zn = cfma(arow[j + 1], make_float2(y2.z, y2.w), zn);
+            }
+          }
         }
       }
       __syncwarp();
