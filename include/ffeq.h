@@ -80,7 +80,8 @@ typedef enum {
 
 typedef enum { FFEQ_PD = 0, FFEQ_FD = 1 } ffeq_arch;
 /* Arithmetic of the local preprocessing (G_c, y_c^MRC); the solve and fusion
- * are FP32 in every mode.
+ * are FP32 in every mode.  FP32, TF32X3 and FP16X3 problems may run one fused
+ * FP32 kernel where it is the faster one (shapes 0 and 1 of the tuning below).
  *   FFEQ_FP32    FP32 on the CUDA cores.
  *   FFEQ_TF32X3  tensor cores, each FP32 operand split into TF32 hi + lo, three
  *                products accumulated in FP32 (about FP32 accuracy).
@@ -284,7 +285,14 @@ ffeq_status ffeq_fd_optimal_backward(const ffeq_plan* plan, const void* H, const
 /* Launch shape of a plan's contraction kernel (the arithmetic is that of the
  * plan's precision in every shape; with split-K (PD) the shapes differ in how
  * the antennas are split among warps, hence in summation order only):
- *   values[0]  0 = default (5 where it applies, else 1), 1 = 16 warps, one CTA per SM,
+ *   values[0]  0 = default (5 where it applies, else 1, 2 or 4 by the sizes),
+ *              1 = 16 warps, one CTA per SM;
+ *              in both, ffeq_equalize of an FD problem with FFEQ_LMMSE or FFEQ_ZF,
+ *              refine = 0 and FP32, TF32X3 or FP16X3 runs ONE kernel that forms the
+ *              local systems in FP32, solves, fuses and writes the soft outputs
+ *              (the workspace is left untouched) where that measured faster: by
+ *              U, n_sym, B, C and n_sc, FP32 mostly, the split precisions with
+ *              few users or symbols; ffeq_local_preprocess runs the contraction;
  *              2 = 8 warps, two CTAs per SM (half the shared memory each),
  *              3 = BF16X3 only: each staged subcarrier converted once into BF16
  *                  hi/lo planes read with ldmatrix (needs B and B/C multiples of 4);

@@ -393,15 +393,15 @@ ffeq_status ffeq_equalize(const ffeq_plan* plan, const void* H, const void* y, f
 
 namespace {
 
-// FP32 FD problems of several clusters, in the default shape, are equalized by the
-// fused kernel where it is the faster one and a subcarrier fits one CTA's shared
-// memory (ffeq_formed.cu).
+// FP32, TF32x3 and FP16x3 FD problems of several clusters, in the default shape, are
+// equalized by the fused FP32 kernel where it is the faster one and a subcarrier
+// fits one CTA's shared memory (ffeq_formed.cu).
 bool formed_applies(const ffeq_plan* plan) {
   const ffeq_problem& p = plan->p;
-  return p.precision == FFEQ_FP32 && p.refine == 0 &&
+  return p.refine == 0 &&
          (p.equalizer == FFEQ_LMMSE || p.equalizer == FFEQ_ZF) &&
          (plan->gram_variant == ffeq::kGramAuto || plan->gram_variant == ffeq::kGram16) &&
-         ffeq::equalize_formed_fits(p.B, p.U, p.n_sym, plan->Ceff, p.n_sc);
+         ffeq::equalize_formed_fits(p.precision, p.B, p.U, p.n_sym, plan->Ceff, p.n_sc);
 }
 
 ffeq_status equalize_impl(const ffeq_plan* plan, const void* H, const void* y, float N0, float Es, void* z,

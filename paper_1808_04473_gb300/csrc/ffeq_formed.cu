@@ -1,4 +1,4 @@
-// Fused FP32 equalization of FD problems (L-MMSE and ZF): one launch from H and y
+// Fused equalization of FD problems in FP32 (L-MMSE and ZF): one launch from H and y
 // to z, sigma^2 and LLRs.
 //
 // A CTA stages one subcarrier and a lane group per cluster forms [G_c + rho I |
@@ -174,9 +174,24 @@ cudaError_t launch_nrc(const FormedParams& p, cudaStream_t stream) {
 // two or three clusters of 32 users leave too few warps per CTA for the contraction (C = 2,
 // S = 128, 300 x 14: 48 -> 72), as those of 16 users and 16 right-hand sides do where an
 // SM has less than two subcarriers (U = 16, C = 2, 64 x 14: 16.6 -> 20.6).
-bool equalize_formed_fits(int B, int U, int n_sym, int C, int n_sc) {
+//
+// TF32x3 and FP16x3 problems run here too where the tensor-core contraction and
+// the solve measured slower (FP32 is at least as accurate: every product rounds
+// once to 24 bits, and nothing is split).  BF16x3 does not: its results are its own.
+//   TF32x3: U = 16, C = 8, 1200 x 3: 56 -> 35; 1200 x 7: 59 -> 41; U = 10, 1200 x 14: 64 -> 47;
+//   U = 32, C = 8, 1200 x 3: 178 -> 133; not U = 14, C = 5, B = 250, 600 x 14 (37 -> 41).
+//   FP16x3: U = 12, C = 16, 800 x 8: 51 -> 37; U = 5, C = 2, 300 x 7: 23 -> 10; U = 11, C = 5,
+//   B = 120, 625 x 13: 33 -> 23; not U = 16, C = 8, 1200 x 14 (46 -> 62).
+bool equalize_formed_fits(int precision, int B, int U, int n_sym, int C, int n_sc) {
   if (C < 2 || (U > 16 && (n_sym > 8 || C < 4))) return false;
   if (U > 8 && n_sym > 8 && C < 4 && n_sc < 2 * 152) return false;
+  if (precision == FFEQ_TF32X3) {
+    if (U > 16 ? n_sym > 4 : (U > 12 && n_sym > 8 && B > 128)) return false;
+  } else if (precision == FFEQ_FP16X3) {
+    if (U > 16 || (n_sym > 8 && B > 128) || (U > 8 && C < 4)) return false;
+  } else if (precision != FFEQ_FP32) {
+    return false;
+  }
   const int UP = padded_users(U), NRC = n_sym <= 4 ? 1 : (n_sym <= 8 ? 2 : 4);
   return 16 + formed_staged_bytes(B, U + n_sym) + static_cast<size_t>(C) * (4 * NRC * UP + UP / 2) * 8 <= 227 * 1024;   // bytes() at most
 }

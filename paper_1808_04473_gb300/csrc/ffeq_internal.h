@@ -148,7 +148,7 @@ struct FormedParams {
   int cl_off[kMaxClusters + 1];
 };
 // Whether that launch applies and is the faster one.
-bool equalize_formed_fits(int B, int U, int n_sym, int C, int n_sc);
+bool equalize_formed_fits(int precision, int B, int U, int n_sym, int C, int n_sc);
 cudaError_t launch_equalize_formed(const FormedParams& p, cudaStream_t stream);
 
 // Status word of a system between the solve and its refinement (fails): the
