@@ -131,6 +131,33 @@ int gram_stages(int precision, int B, int U, int n_sym, int Ceff, bool bulk) {
   return gram_stages_fit(c.stage_elems, static_cast<size_t>(c.slots) * c.slot_elems * 8, bulk);
 }
 
+// Default shape of a contraction that the streamed kernel does not take: several
+// small CTAs per SM where they fit and there are subcarriers enough for them,
+// because a CTA takes its subcarriers one at a time and its waits, barriers and
+// split-K reduction are exposed unless another CTA's products cover them.  Measured
+// (us a call, 16 warps -> this): PD TF32x3 U = 6, B = 96, 3000 x 4: 58 -> 27 (4 warps x 3);
+// PD TF32x3 U = 12, B = 100, 333 x 7: 20.6 -> 16.6 (4 x 3); FD BF16x3 U = 20, C = 5,
+// 800 x 6: 88 -> 78 (4 x 3, 10 of 16 warps busy before); PD TF32x3 U = 16, 1200 x 14: 55 -> 47
+// (8 x 2; 4 x 3 with one stage 49); PD FP32 U = 16, 1200 x 14: 60 -> 53 (8 x 2).  FD with
+// items for all 16 warps gains nothing (TF32x3 C = 8: 135 -> 136) and keeps them, as do
+// 100 subcarriers (14.3 -> 16.4) and, before 8 x 2 has two rounds for every CTA, 400
+// (PD TF32x3 U = 28: 51 -> 54).
+static int default_shape(const GramParams& p, int precision) {
+  constexpr int kSms = 152;
+  if (!p.bulk || p.n_sc < 2 * kSms || precision == FFEQ_FP16X3) return kGram16;
+  auto stages_of = [&](int variant) {
+    const GramCaps c = gram_instance_caps(precision, p.B, p.U, p.n_sym, p.Ceff, variant);
+    return gram_stages_fit(c.stage_elems, static_cast<size_t>(c.slots) * c.slot_elems * 8, true,
+                           gram_smem_budget(variant));
+  };
+  if (precision != FFEQ_FP32) {
+    const int fit = stages_of(kGram4x3);
+    const int items = p.Ceff * ((p.U + p.n_sym + 15) / 16);
+    if (fit >= 2 || (fit == 1 && p.Ceff > 1 && items % 16 != 0)) return kGram4x3;
+  }
+  return p.Ceff == 1 && p.n_sc >= 4 * kSms && stages_of(kGram8x2) >= 1 ? kGram8x2 : kGram16;
+}
+
 bool gram_configure(GramParams& p, int precision, int variant, int stages) {
   p.n_units = p.n_sc;
   p.desc = nullptr;
@@ -139,9 +166,9 @@ bool gram_configure(GramParams& p, int precision, int variant, int stages) {
   p.lim = BatchLimits{};
   p.grid_cap = 0;
   const bool stream_ok = p.cl_uniform && gram_stream_eligible(precision, p.B, p.U, p.n_sym, p.Ceff);
-  // Default: the streamed shape where it applies (16-byte aligned inputs),
-  // else 16 warps.
-  if (variant == kGramAuto) variant = stream_ok && p.bulk ? kGramStream : kGram16;
+  // Default: the streamed shape where it applies (16-byte aligned inputs).
+  if (variant == kGramAuto)
+    variant = stream_ok && p.bulk ? kGramStream : (stages == 0 ? default_shape(p, precision) : kGram16);
   if (variant < kGram16 || variant > kGramVariantMax) return false;
   if (variant == kGramFused) {
     // The contraction of the fused shape is the streamed one with a ring of 2
