@@ -84,12 +84,12 @@ namespace {
 // Contraction shape of an instance: two CTAs of 8 warps per SM where one staged
 // unit fits half of the shared memory, so that one unit's waits, barriers and
 // reduction overlap the other's products (a CTA takes its units one at a time);
-// one of 16 warps where it does not fit, or where the batch has fewer than two
+// one of 16 warps where it does not fit, or where the batch has fewer than three
 // units per SM and a unit's own latency counts.  4096 instances of 4 to 32 users,
-// BF16x3: FD 387 -> 342 us, PD 224 -> 168; FP32 FD 416 -> 377; 100 instances: 53
-// with 16 warps, 56 with 8.
+// BF16x3: FD 387 -> 342 us, PD 224 -> 168; FP32 FD 416 -> 377; 659 instances: 61 -> 54;
+// 326 instances: 42.6 with 16 warps, 43.8 with 8; 100: 53 and 56.
 int batch_variant(const ffeq_batch_config& cfg, const ffeq_instance& in, long long n_units) {
-  if (n_units < 2 * kSms) return ffeq::kGram16;
+  if (n_units < 3 * kSms) return ffeq::kGram16;
   const int Ceff = cfg.arch == FFEQ_FD ? in.C : 1;
   const ffeq::GramCaps gc =
       ffeq::gram_instance_caps(cfg.precision, in.B, in.U, in.n_sym, Ceff, ffeq::kGram8x2);

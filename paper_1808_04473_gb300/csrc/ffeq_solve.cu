@@ -149,46 +149,52 @@ __device__ void batch_epilogue(const SolveParams& p, const float2* base, const i
 // z = num / den, sigma^2 = s2_scale / den (s2_scale = N0 for the solve, whose
 // denominators are g / A_uu; Es for MRC, whose are Es / sigma_c^2) and the LLRs.
 // System m's fusion area (numerators [n][UP], denominators) is areas + m stride.
-// Outputs are walked in the padded order (n, u < UP), so that the index splits
-// by a constant.  zflag [spc][UP] (MRC, or nullptr): users fused with the
-// N0 -> 0 limit weights, whose variance is 0.
-template <int UP>
+// Outputs are walked in the order (n, u), PADDED over u < UP, so that the index
+// splits by a constant, or over u < U (MRC, whose epilogue is most of its work: a
+// third of the lanes idle with U = 21 costs 6%).  zflag [spc][UP] (MRC, or
+// nullptr): users fused with the N0 -> 0 limit weights, whose variance is 0.
+template <int UP, bool PADDED>
 __device__ __forceinline__ void uniform_epilogue(const SolveParams& p, const float2* areas, int stride,
                                                  const int* fail_sc, int sc0, int U, int NS, int Ceff, float s2_scale,
                                                  const int* zflag = nullptr) {
   const int bits = p.llr_bits, hb = bits / 2;
-  for (int s = 0; s < p.spc; ++s) {
+  // (subcarrier s, output e) of this thread, advanced by the CTA's threads without
+  // a division per output.
+  const int per = (PADDED ? UP : U) * NS, ds = static_cast<int>(blockDim.x) / per, de = static_cast<int>(blockDim.x) - ds * per;
+  int s = threadIdx.x / per, e = threadIdx.x - s * per;
+  for (; s < p.spc && sc0 + s < p.n_sc; s += ds, e += de) {
+    if (e >= per) {
+      e -= per;
+      if (++s >= p.spc || sc0 + s >= p.n_sc) break;
+    }
+    const int n = PADDED ? e / UP : e / U, u = PADDED ? e % UP : e - n * U;
+    if (PADDED && u >= U) continue;
     const int k = sc0 + s;
-    if (k >= p.n_sc) break;
     const float2* sys = areas + static_cast<size_t>(s) * Ceff * stride;
     const bool failed = fail_sc[s] != 0;
-    for (int e = threadIdx.x; e < UP * NS; e += blockDim.x) {
-      const int n = e / UP, u = e % UP;
-      if (u >= U) continue;
-      float2 nm = make_float2(0.f, 0.f);
-      float dn = 0.f;
-      for (int cc = 0; cc < Ceff; ++cc) {
-        nm = cadd(nm, sys[cc * stride + e]);
-        dn += reinterpret_cast<const float*>(sys + cc * stride + kNsymMax * UP)[u];
-      }
-      float2 zz;
-      float s2;
-      if (failed) {
-        zz = make_float2(NAN, NAN);
-        s2 = NAN;
-      } else if (dn > 0.f) {
-        const float rr = rcp_approx(dn);
-        zz = cscale(nm, rr);
-        s2 = (zflag && zflag[s * UP + u]) ? 0.f : s2_scale * rr;
-      } else {
-        zz = make_float2(0.f, 0.f);
-        s2 = INFINITY;
-      }
-      const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
-      p.z[zi] = zz;
-      if (n == 0) p.sigma2[static_cast<size_t>(k) * U + u] = s2;
-      if (bits) symbol_llr_wide(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
+    float2 nm = make_float2(0.f, 0.f);
+    float dn = 0.f;
+    for (int cc = 0; cc < Ceff; ++cc) {
+      nm = cadd(nm, sys[cc * stride + n * UP + u]);
+      dn += reinterpret_cast<const float*>(sys + cc * stride + kNsymMax * UP)[u];
     }
+    float2 zz;
+    float s2;
+    if (failed) {
+      zz = make_float2(NAN, NAN);
+      s2 = NAN;
+    } else if (dn > 0.f) {
+      const float rr = rcp_approx(dn);
+      zz = cscale(nm, rr);
+      s2 = (zflag && zflag[s * UP + u]) ? 0.f : s2_scale * rr;
+    } else {
+      zz = make_float2(0.f, 0.f);
+      s2 = INFINITY;
+    }
+    const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
+    p.z[zi] = zz;
+    if (n == 0) p.sigma2[static_cast<size_t>(k) * U + u] = s2;
+    if (bits) symbol_llr_wide(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
   }
 }
 
@@ -246,7 +252,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? (UP <= 16 ? 5 : 3) : 1) so
   }
   if (p.Xs) return;   // the refinement kernel fuses and writes the outputs
   __syncthreads();
-  uniform_epilogue<UP>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
+  uniform_epilogue<UP, true>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
 }
 
 template <int UP, int NRC, int MAXT>
@@ -817,7 +823,7 @@ __global__ void __launch_bounds__(512) mrc_fuse_kernel(const SolveParams p) {
     Dn[i] = w;
   }
   __syncthreads();
-  uniform_epilogue<UP>(p, base + Lay::kRow, Lay::kMat, fail_sc, sc0, U, NS, Ceff, p.Es, zflag);
+  uniform_epilogue<UP, false>(p, base + Lay::kRow, Lay::kMat, fail_sc, sc0, U, NS, Ceff, p.Es, zflag);
 }
 
 template <int UP>
@@ -952,11 +958,11 @@ cudaError_t launch_mrc_batch(const SolveParams& p, cudaStream_t stream) {
 
 }  // namespace
 
-// PD (one system per subcarrier) with 8 < U < 16: a full warp per system (two
-// lanes per row) and 4 subcarriers per CTA, for more warps in flight; PD with
-// U = 8, 16 or 32 (solve_full_kernel): 2 subcarriers per CTA, one lane per row
-// (measured faster than two lanes per row: half the instructions per system);
-// FD: the C systems of one subcarrier in one CTA, UP lanes each.
+// Subcarriers per CTA of the row kernel and of MRC, which a plan's limits count too
+// (the tile kernel takes its own): FD one, its C systems in one CTA with UP lanes
+// each; PD two where the users fill the lane group (one lane per row, measured
+// faster than two: half the instructions per system), else as many as made 128
+// lanes when a row of 9 to 15 users took two.
 static int lanes_per_row(int U, int Ceff) { return (Ceff == 1 && padded_users(U) == 16 && U != 16) ? 2 : 1; }
 
 int solve_subcarriers_per_cta(int U, int Ceff) {
