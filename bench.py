@@ -826,7 +826,7 @@ def uneven_line(R, K, warmup, precision, sampler=None):
         "tuning": {("pd" if a == ffeq.PD else "fd"): ffeq.ffeq_batch_get_tuning(r["b"]) for a, r in runs.items()},
         "schedule": {"mode": "concurrent" if concurrent else "sequential",
                      "chosen_by": "timing PD and FD in sequence and as two graph branches"},
-        "roofline": {"kernel": "whole step (memset + per-group gram_kernel and solve_fuse_kernel)", "bound": "hbm",
+        "roofline": {"kernel": "whole step (memset + per-group gram_kernel and solve_batch_kernel)", "bound": "hbm",
                      "achieved": achieved, "peak": hbm_peak, "peak_source": f"{peak_src} (STREAM-style copy)",
                      "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": None,
                      "algorithmic_bytes_per_step": alg},

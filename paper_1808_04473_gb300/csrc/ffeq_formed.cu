@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kThreads, 2) equalize_formed_kernel(const Form
       const int S = p.cl_uniform ? B / C : 0;
       const int b0 = p.cl_uniform ? c * S : p.cl_off[c], b1 = p.cl_uniform ? b0 + S : p.cl_off[c + 1];
       float re[F::RPL][NC], im[F::RPL][NC], rs[F::RPL];
-      formed_tile<UP, NRC, true>(Ws, RS, U, NS, b0, b1, r, q, valid, 0.f, re, im);
+      formed_tile<UP, NRC, true, true>(Ws, RS, U, NS, b0, b1, r, q, valid, 0.f, re, im);
       if (at_once) __syncthreads();   // one pass: the staged rows are no longer read
       unsigned zero_diag = 0;   // users this cluster cannot see (G_ii = 0), one bit per row of the lane
 #pragma unroll

@@ -16,8 +16,8 @@
 // cyclic rows and the stride (4 floats past a multiple of 32) put the rows one
 // load phase reads in different banks, and natural rows stage with 16-byte
 // copies (4-byte ones before, to turn the rows around).  Measured on 8192
-// subcarriers, B = 128, U = 16, C = 8, one symbol (before -> after): training
-// forward 175 -> 126 us, backward 211 -> 146, optimal adjoint 352 -> 292.  What
+// subcarriers, B = 128, U = 16, C = 8, one symbol (before -> after): training step
+// 407 -> 296 us (282 with HALF below), optimal adjoint 352 -> 292.  What
 // bounds them now: issue (72-74%), FMA pipe 39-48%, 16 warps per SM.
 //
 // Scalar FMAs: a paired FMA takes two cycles of the pipe (67 against 68 TFLOP/s
@@ -82,8 +82,14 @@ __device__ __forceinline__ void formed_wait() {
 // rows: re/im[i][j] = sum_b conj(H[r + RL i][b]) W[col][b], columns j < CA users,
 // then (WITH_Y) NRC symbols, in antenna order.  Padding rows and columns are
 // identity; a lane of an invalid group holds an identity system.  Every lane of
-// the warp takes part.
-template <int UP, int NRC, bool WITH_Y>
+// the warp takes part.  G_c is Hermitian, so with four row lanes the entries right
+// of the tile diagonal come from lane (q, r): HALF takes their conjugates, whose
+// imaginary parts add the two products of an antenna in the other order; otherwise
+// only the real parts (the same bits).  The training pair does the latter, so that
+// its X and G_b keep their bits: the gradient of the regularizers cancels 25- to
+// 45-fold over the subcarriers, and another rounding of the ill-conditioned solves
+// moves it by a few 1e-6 either way.
+template <int UP, int NRC, bool WITH_Y, bool HALF>
 __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int NS, int b0, int b1, int r, int q,
                                             bool valid, float rho,
                                             float (&re)[FormedShape<UP>::RPL][FormedShape<UP>::CA + NRC],
@@ -106,13 +112,14 @@ __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int 
   for (int i = 0; i < F::RPL; ++i)
 #pragma unroll
     for (int j = 0; j < NC; ++j) re[i][j] = im[i][j] = 0.f;
-  // G_c is Hermitian: with four row lanes the entries right of the tile diagonal
-  // are the conjugates of entries of lane (q, r), fetched afterwards.
   constexpr bool kHalf = F::RL == 4;
   auto acc = [&](int i, int j, float hr, float hi, float wr, float wi) {   // conj(h) w
-    if (kHalf && j < F::CA && j > i) return;
-    re[i][j] = fmaf(hr, wr, re[i][j]);
-    re[i][j] = fmaf(hi, wi, re[i][j]);
+    const bool far = kHalf && j < F::CA && j > i;
+    if (HALF && far) return;
+    if (!far) {
+      re[i][j] = fmaf(hr, wr, re[i][j]);
+      re[i][j] = fmaf(hi, wi, re[i][j]);
+    }
     im[i][j] = fmaf(hr, wi, im[i][j]);
     im[i][j] = fmaf(-hi, wr, im[i][j]);
   };
@@ -150,7 +157,7 @@ __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int 
 #pragma unroll
       for (int j = i + 1; j < F::CA; ++j) {
         re[i][j] = __shfl_sync(kFullMask, re[j][i], 4 * q + r, F::GL);
-        im[i][j] = -__shfl_sync(kFullMask, im[j][i], 4 * q + r, F::GL);
+        if (HALF) im[i][j] = -__shfl_sync(kFullMask, im[j][i], 4 * q + r, F::GL);
       }
     }
   }

@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kFormedThreads, 2) train_forward_fused_kernel(
       int b0, b1;
       cluster_range(p, c, b0, b1);
       float re[F::RPL][F::CA + NRC], im[F::RPL][F::CA + NRC], rs[F::RPL];
-      formed_tile<UP, NRC, true>(Ws, RS, U, NS, b0, b1, r, q, valid, p.rho_c[c], re, im);
+      formed_tile<UP, NRC, true, false>(Ws, RS, U, NS, b0, b1, r, q, valid, p.rho_c[c], re, im);
       const int fail = formed_sweep<UP, NRC, false>(re, im, U, r, q, rs);
       if (valid && gl == 0 && fail) atomicOr(fail_any, 1);
       if (valid) {
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(kFormedThreads, 2) train_backward_fused_kernel
         xr[i] = real ? p.X[off + q * U + u] : make_float2(0.f, 0.f);
       }
       float re[F::RPL][F::CA + NRC], im[F::RPL][F::CA + NRC], rs[F::RPL];
-      formed_tile<UP, NRC, false>(Ws, RS, U, NS, b0, b1, r, q, valid, p.rho_c[c], re, im);
+      formed_tile<UP, NRC, false, false>(Ws, RS, U, NS, b0, b1, r, q, valid, p.rho_c[c], re, im);
 #pragma unroll
       for (int i = 0; i < F::RPL; ++i) {
         const int u = r + F::RL * i;
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kFormedThreads, 2) train_optimal_fused_kernel(
       int b0, b1;
       cluster_range(p, c, b0, b1);
       float re[F::RPL][F::CA + NRC], im[F::RPL][F::CA + NRC], rs[F::RPL];
-      formed_tile<UP, NRC, true>(Ws, RS, U, NS, b0, b1, r, q, valid, rho, re, im);
+      formed_tile<UP, NRC, true, true>(Ws, RS, U, NS, b0, b1, r, q, valid, rho, re, im);
       const int fail = formed_sweep<UP, NRC, true>(re, im, U, r, q, rs);
       if (valid && gl == 0 && fail) atomicOr(fail_any, 1);
 #pragma unroll
