@@ -1,63 +1,22 @@
-// Register-resident Gauss-Jordan sweep shared by the solve kernels.
+// Register-resident Gauss-Jordan sweeps with one row per lane, shared by the solve
+// kernels (ffeq_tile.cuh and ffeq_formed.cuh hold the register tiles).
 //
 // A group of UP lanes (UP a power of two <= 32) holds one Hermitian positive
-// definite system [M | R]: lane i keeps row i in aug[0..W) with M in the first
-// UP columns and R in the remaining W - UP.  Each step k scales the pivot row by
-// 1/p_k, broadcasts it through shared memory (rowbuf, W complex, 16-byte
-// aligned) and eliminates it from every other row; the row is rotated left by
-// one so the pivot column is always aug[0] and the new inverse column lands in
-// aug[W-1].  All register indices are compile-time constants while the step
-// loop is a runtime loop.  On return, lane i holds row i of M^{-1} R in
-// aug[0 .. W-UP) and row i of M^{-1} in aug[W-UP .. W).  The pivots p_k are the
-// Schur complements of M (the squared diagonal of its Cholesky factor); the
-// return value is the 1-based index of the first pivot that is not positive, or
-// 0.  `writer` is false for lanes that must not write rowbuf (spare lanes).
+// definite system [M | R]: lane i keeps row i with M in the first UP columns and R
+// in the remaining W - UP.  Step k broadcasts the pivot row through shared memory
+// and eliminates it from every other row; the columns are rotated left, so that the
+// pivot column sits at a compile-time index while the step loop is a runtime loop,
+// and the new inverse columns land at the end.  On return, lane i holds row i of
+// M^{-1} R in columns 0 .. W-UP-1 and row i of M^{-1} in columns W-UP .. W-1.  The
+// pivots p_k are the Schur complements of M (the squared diagonal of its Cholesky
+// factor); the return value is the 1-based index of the first pivot that is not
+// positive, or 0.  `writer` is false for lanes that must not write rowbuf (spare
+// lanes).
 #pragma once
 
 #include "ffeq_device.cuh"
 
 namespace ffeq {
-
-template <int UP, int W>
-__device__ __forceinline__ int gj_sweep_rotating(float2 (&aug)[W], float2* rowbuf, int i, bool writer) {
-  static_assert(W % 2 == 0, "row width must be even");
-  int fail = 0;
-#pragma unroll 1
-  for (int k = 0; k < UP; ++k) {
-    const float piv = __shfl_sync(kFullMask, aug[0].x, k, UP);
-    const bool ok = piv > 0.f;
-    if (!ok && fail == 0) fail = k + 1;
-    const float r = 1.f / (ok ? piv : 1.f);
-    if (i == k && writer) {
-      // Scaled pivot row in the rotated layout: [aug[1..W-1] * r, r].
-#pragma unroll
-      for (int j = 0; j < W; j += 2) {
-        const float2 v0 = j + 1 < W ? cscale(aug[j + 1], r) : make_float2(r, 0.f);
-        const float2 v1 = j + 2 < W ? cscale(aug[j + 2], r) : make_float2(r, 0.f);
-        *reinterpret_cast<float4*>(rowbuf + j) = make_float4(v0.x, v0.y, v1.x, v1.y);
-      }
-    }
-    __syncwarp();
-    const float2 f = aug[0];
-    if (i == k) {
-#pragma unroll
-      for (int j = 0; j < W; j += 2) {
-        const float4 q = *reinterpret_cast<const float4*>(rowbuf + j);
-        aug[j] = make_float2(q.x, q.y);
-        aug[j + 1] = make_float2(q.z, q.w);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < W; j += 2) {
-        const float4 q = *reinterpret_cast<const float4*>(rowbuf + j);
-        aug[j] = j + 1 < W ? cfms(f, make_float2(q.x, q.y), aug[j + 1]) : make_float2(-f.x * r, -f.y * r);
-        aug[j + 1] = j + 2 < W ? cfms(f, make_float2(q.z, q.w), aug[j + 2]) : make_float2(-f.x * r, -f.y * r);
-      }
-    }
-    __syncwarp();
-  }
-  return fail;
-}
 
 // One element of the deferred-scaling elimination, shared by every sweep so
 // that all lane layouts round identically:
@@ -89,8 +48,7 @@ __device__ __forceinline__ void gj_rotate_padding(float2 (&rp)[W / 2], float2 (&
 
 // Gauss-Jordan sweep with deferred row scaling and paired FMAs.
 //
-// Same system and result layout as gj_sweep_rotating, held as pairs of
-// adjacent columns: rp[m] = (re col 2m, re col 2m+1), ip[m] likewise for the
+// The system is held as pairs of adjacent columns: rp[m] = (re col 2m, re col 2m+1), ip[m] likewise for the
 // imaginary parts (lane i = row i).  At step k the pivot row is broadcast
 // UNSCALED (its pivot-column entry replaced by 1, the identity column it turns
 // into) together with the pivot p_k, and every other row does new = base - g q
@@ -320,60 +278,6 @@ __device__ __forceinline__ int gj_sweep_block2(float2 (&rp)[W / 2], float2 (&ip)
   }
   gj_rotate_padding<W>(rp, ip, UP - steps);
   __syncwarp();   // the areas may be reused after the sweep
-  scale = my_r;
-  return fail;
-}
-
-// The same sweep (deferred scaling, two steps per trip, rotation by two, one
-// broadcast buffer per step) on interleaved complex registers with scalar FMAs
-// (gj_update), which rounds exactly like gj_sweep_pairs.  rowbuf: 2 (2W + 4)
-// floats, 16-byte aligned.
-template <int UP, int W>
-__device__ __forceinline__ int gj_sweep_deferred(float2 (&aug)[W], float* rowbuf, int i, bool writer,
-                                                 float& scale) {
-  static_assert(W % 2 == 0 && UP % 2 == 0, "sweep needs even W and UP");
-  constexpr int kBuf = 2 * W + 4;          // W complex, then the pivot (padded to 16 bytes)
-  int fail = 0;
-  float my_r = 1.f;
-#pragma unroll 1
-  for (int k = 0; k < UP; k += 2) {
-    static_for<2>([&](auto sc) {
-      constexpr int s = decltype(sc)::value;   // pivot column of this step
-      float* buf = rowbuf + s * kBuf;
-      const int kk = k + s;
-      const bool me = i == kk;
-      if (me && writer) {
-#pragma unroll
-        for (int j = 0; j < W; j += 2) {
-          const float2 a = j == s ? make_float2(1.f, 0.f) : aug[j];
-          const float2 b = j + 1 == s ? make_float2(1.f, 0.f) : aug[j + 1];
-          *reinterpret_cast<float4*>(buf + 2 * j) = make_float4(a.x, a.y, b.x, b.y);
-        }
-        buf[2 * W] = aug[s].x;
-      }
-      __syncwarp();
-      const float piv = buf[2 * W];
-      const bool ok = piv > 0.f;
-      if (!ok && fail == 0) fail = kk + 1;
-      const float r = rcp_approx(ok ? piv : 1.f);
-      if (me) my_r = r;
-      const float2 gg = me ? make_float2(0.f, 0.f) : make_float2(aug[s].x * r, aug[s].y * r);
-      const float dlt = me ? 1.f : 0.f;
-      float2 nw[W];
-#pragma unroll
-      for (int j = 0; j < W; j += 2) {
-        const float4 q = *reinterpret_cast<const float4*>(buf + 2 * j);
-        const float2 b0 = j == s ? make_float2(dlt, 0.f) : aug[j];
-        const float2 b1 = j + 1 == s ? make_float2(dlt, 0.f) : aug[j + 1];
-        const int d = s == 1 ? (j + W - 2) % W : j;   // after the second step, rotate left by two
-        nw[d] = gj_update(gg, make_float2(q.x, q.y), b0);
-        nw[d + 1] = gj_update(gg, make_float2(q.z, q.w), b1);
-      }
-#pragma unroll
-      for (int j = 0; j < W; ++j) aug[j] = nw[j];
-    });
-  }
-  __syncwarp();   // the buffers may be reused after the sweep
   scale = my_r;
   return fail;
 }
