@@ -47,7 +47,17 @@ __device__ __forceinline__ void ld2(const float2* __restrict__ row, int a, int k
 // One warp: rows [16 mtile, 16 mtile + 16) of D over antennas [k0, k1) (H rows
 // then Y rows; rows >= Mrows read row 0 and are dropped), NX = UP/8 tiles of 8
 // users for the real parts (x) and NX for the imaginary parts (r).
-template <int UP, int MODE, typename Out>
+//
+// EMPTY (TF32x3 with fewer than 16 warps): the MMA accumulators start from zero
+// at every k-step and are added to FP32 sums of Re D and Im D.  An MMA does not
+// round its sums to nearest, so the error grows with the k-steps chained in one
+// accumulator; fewer warps make fewer K-parts of more k-steps each.  RMS error of
+// sigma^2 against 64 bits, PD, ZF, 16 warps / 4 or 8 warps chained / emptied:
+// B = 100, U = 12: 2.5e-7 / 5.7e-7 / 2.0e-7; B = 256, U = 8: 1.7e-7 / 5.1e-7 / 1.4e-7.
+// Ten paired additions per 8 users and k-step: 0-1% of a PD call with up to 12
+// users, 3% with 16 (1200 x 14: 45.3 -> 46.7 us), up to 7% of an FD call with 24
+// (C = 2, 800 x 9: 72.8 -> 78.1 us).
+template <int UP, int MODE, bool EMPTY, typename Out>
 __device__ __forceinline__ void tc_tiles(const float2* __restrict__ Ws, int RS, int Mrows, int U, int k0, int k1,
                                          bool vec, int lane, int mtile, Out out) {
   constexpr int NX = UP / 8;
@@ -59,12 +69,14 @@ __device__ __forceinline__ void tc_tiles(const float2* __restrict__ Ws, int RS, 
 
   // Gauss's three-product complex multiply: with T1 = A_re B_re, T2 = A_im B_im and
   // T3 = (A_re + A_im)(B_re - B_im), Re D = T1 + T2 and Im D = T3 - T1 + T2.
-  // acc[i][3j + q] holds T_{q+1} of user tile j.
-  float acc[MTMAX][3 * NX][4];
+  // acc[i][3j + q] holds T_{q+1} of user tile j; EMPTY: acc[i][2j] holds Re D and
+  // acc[i][2j + 1] Im D.
+  constexpr int NA = EMPTY ? 2 : 3;
+  float acc[MTMAX][NA * NX][4];
 #pragma unroll
   for (int i = 0; i < MTMAX; ++i)
 #pragma unroll
-    for (int j = 0; j < 3 * NX; ++j)
+    for (int j = 0; j < NA * NX; ++j)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
 
@@ -141,22 +153,53 @@ __device__ __forceinline__ void tc_tiles(const float2* __restrict__ Ws, int RS, 
             split_pair<MODE>(w0[q].x + w0[q].y, w1[q].x + w1[q].y, as_h[q], as_l[q]);
           }
         }
-        // Issue order: one split product (A_lo B_hi, A_hi B_lo, A_hi B_hi) at a
-        // time over every accumulator tile, so consecutive MMAs never wait on
-        // each other.
-#pragma unroll
-        for (int prod = 0; prod < 3; ++prod) {
-          const uint32_t(&ar)[4] = prod == 0 ? are_l : are_h;
-          const uint32_t(&ai)[4] = prod == 0 ? aim_l : aim_h;
-          const uint32_t(&as)[4] = prod == 0 ? as_l : as_h;
+        if constexpr (EMPTY) {
 #pragma unroll
           for (int j = 0; j < NX; ++j) {
-            mma_any<MODE>(acc[i][3 * j], ar, prod == 1 ? bre_l[j][0] : bre_h[j][0],
-                          prod == 1 ? bre_l[j][1] : bre_h[j][1]);
-            mma_any<MODE>(acc[i][3 * j + 1], ai, prod == 1 ? bim_l[j][0] : bim_h[j][0],
-                          prod == 1 ? bim_l[j][1] : bim_h[j][1]);
-            mma_any<MODE>(acc[i][3 * j + 2], as, prod == 1 ? bd_l[j][0] : bd_h[j][0],
-                          prod == 1 ? bd_l[j][1] : bd_h[j][1]);
+            float t[3][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[0][q] = t[1][q] = t[2][q] = 0.f;
+#pragma unroll
+            for (int prod = 0; prod < 3; ++prod) {
+              mma_any<MODE>(t[0], prod == 0 ? are_l : are_h, prod == 1 ? bre_l[j][0] : bre_h[j][0],
+                            prod == 1 ? bre_l[j][1] : bre_h[j][1]);
+              mma_any<MODE>(t[1], prod == 0 ? aim_l : aim_h, prod == 1 ? bim_l[j][0] : bim_h[j][0],
+                            prod == 1 ? bim_l[j][1] : bim_h[j][1]);
+              mma_any<MODE>(t[2], prod == 0 ? as_l : as_h, prod == 1 ? bd_l[j][0] : bd_h[j][0],
+                            prod == 1 ? bd_l[j][1] : bd_h[j][1]);
+            }
+            float* re = acc[i][2 * j];
+            float* im = acc[i][2 * j + 1];
+#pragma unroll
+            for (int q = 0; q < 4; q += 2) {   // two entries per paired addition
+              const float2 t1 = make_float2(t[0][q], t[0][q + 1]), t2 = make_float2(t[1][q], t[1][q + 1]);
+              const float2 d3 = __ffma2_rn(t1, make_float2(-1.f, -1.f), make_float2(t[2][q], t[2][q + 1]));
+              const float2 r = __fadd2_rn(make_float2(re[q], re[q + 1]), __fadd2_rn(t1, t2));
+              const float2 m = __fadd2_rn(make_float2(im[q], im[q + 1]), __fadd2_rn(d3, t2));
+              re[q] = r.x;
+              re[q + 1] = r.y;
+              im[q] = m.x;
+              im[q + 1] = m.y;
+            }
+          }
+        } else {
+          // Issue order: one split product (A_lo B_hi, A_hi B_lo, A_hi B_hi) at a
+          // time over every accumulator tile, so consecutive MMAs never wait on
+          // each other.
+#pragma unroll
+          for (int prod = 0; prod < 3; ++prod) {
+            const uint32_t(&ar)[4] = prod == 0 ? are_l : are_h;
+            const uint32_t(&ai)[4] = prod == 0 ? aim_l : aim_h;
+            const uint32_t(&as)[4] = prod == 0 ? as_l : as_h;
+#pragma unroll
+            for (int j = 0; j < NX; ++j) {
+              mma_any<MODE>(acc[i][3 * j], ar, prod == 1 ? bre_l[j][0] : bre_h[j][0],
+                            prod == 1 ? bre_l[j][1] : bre_h[j][1]);
+              mma_any<MODE>(acc[i][3 * j + 1], ai, prod == 1 ? bim_l[j][0] : bim_h[j][0],
+                            prod == 1 ? bim_l[j][1] : bim_h[j][1]);
+              mma_any<MODE>(acc[i][3 * j + 2], as, prod == 1 ? bd_l[j][0] : bd_h[j][0],
+                            prod == 1 ? bd_l[j][1] : bd_h[j][1]);
+            }
           }
         }
       }
@@ -174,12 +217,18 @@ __device__ __forceinline__ void tc_tiles(const float2* __restrict__ Ws, int RS, 
           const int m = mbase + i * 16 + g + 8 * h;
           const int u = j * 8 + 2 * t;
           if (m < Mrows && u < U) {
-            const float* t1 = acc[i][3 * j];
-            const float* t2 = acc[i][3 * j + 1];
-            const float* t3 = acc[i][3 * j + 2];
             const int q0 = 2 * h, q1 = 2 * h + 1;
-            out(m, u, make_float2(t1[q0] + t2[q0], t3[q0] - t1[q0] + t2[q0]),
-                make_float2(t1[q1] + t2[q1], t3[q1] - t1[q1] + t2[q1]), u + 1 < U);
+            if constexpr (EMPTY) {
+              const float* re = acc[i][2 * j];
+              const float* im = acc[i][2 * j + 1];
+              out(m, u, make_float2(re[q0], im[q0]), make_float2(re[q1], im[q1]), u + 1 < U);
+            } else {
+              const float* t1 = acc[i][3 * j];
+              const float* t2 = acc[i][3 * j + 1];
+              const float* t3 = acc[i][3 * j + 2];
+              out(m, u, make_float2(t1[q0] + t2[q0], t3[q0] - t1[q0] + t2[q0]),
+                  make_float2(t1[q1] + t2[q1], t3[q1] - t1[q1] + t2[q1]), u + 1 < U);
+            }
           }
         }
       }
@@ -197,7 +246,7 @@ struct TensorSplit {
   template <int UP, typename Out>
   __device__ __forceinline__ static void run(const float2* __restrict__ Ws, int RS, int Mrows, int U, int k0,
                                              int k1, bool vec, int lane, int mt, Out out) {
-    tc_tiles<UP, MODE>(Ws, RS, Mrows, U, k0, k1, vec, lane, mt, out);
+    tc_tiles<UP, MODE, MODE == kTf32x3 && (WARPS < 16)>(Ws, RS, Mrows, U, k0, k1, vec, lane, mt, out);
   }
 };
 
