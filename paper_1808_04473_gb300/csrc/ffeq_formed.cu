@@ -20,10 +20,24 @@ namespace {
 
 constexpr int kThreads = 256;   // at most
 
+// How a cluster's antennas are added up.  With five clusters or more, in one chain.
+// With two to four, in parts, eight for the subcarrier as in the contraction launch,
+// because the error of a chain grows with its antennas: rms of z against 64 bits, two
+// clusters of 16 / 128 / 512 antennas, contraction launch 1.4e-7 / 1.3e-7 / 1.6e-7,
+// one chain 1.7e-7 / 2.5e-7 / 4.4e-7, parts 1.3e-7 / 1.2e-7 / 1.5e-7.  A lane takes its
+// parts one after another (kSerial), or each part has a lane group (kGroups).
+enum Adding { kOneChain, kSerial, kGroups };
+
 template <int UP, int NRC>
+constexpr int kTileFloats = 2 * FormedShape<UP>::RPL * (FormedShape<UP>::CA + NRC);   // a lane holds
+
+template <int UP, int NRC, Adding ADD>
 struct FormedEqLayout {
   static constexpr int NR = 4 * NRC;
   static constexpr int AREA = NR * UP + UP / 2;   // float2 per cluster: numerators [NR][UP], denominators [UP]
+  static constexpr int TILE = kTileFloats<UP, NRC>;
+  __host__ __device__ static int parts(int C) { return ADD == kOneChain ? 1 : 8 / C; }
+  __host__ __device__ static int group_parts(int C) { return ADD == kGroups ? parts(C) : 1; }
   static int groups(int C) {
     const int most = kThreads / FormedShape<UP>::GL;
     return C < most ? C : most;
@@ -34,21 +48,23 @@ struct FormedEqLayout {
   __host__ __device__ static size_t areas(int B, int rows, bool at_once) {
     return 16 + (at_once ? 0 : formed_staged_bytes(B, rows));
   }
+  // After them the tiles of the parts past the first ([part][cluster][TILE][GL]).
   static size_t bytes(int B, int U, int n_sym, int C) {
     const size_t rows = formed_staged_bytes(B, U + n_sym), terms = static_cast<size_t>(C) * AREA * sizeof(float2);
-    return 16 + (groups(C) == C ? (rows > terms ? rows : terms) : rows + terms);
+    const size_t tiles = static_cast<size_t>(group_parts(C) - 1) * C * TILE * FormedShape<UP>::GL * sizeof(float);
+    return 16 + (groups(C) == C ? (rows > terms + tiles ? rows : terms + tiles) : rows + terms);
   }
   static int threads(int B, int C) {
-    const int t = groups(C) * FormedShape<UP>::GL, w = B < 128 ? B : 128;
+    const int t = groups(C) * group_parts(C) * FormedShape<UP>::GL, w = B < 128 ? B : 128;
     return (((t > w ? t : w) + 31) / 32) * 32;
   }
 };
 
-template <int UP, int NRC>
+template <int UP, int NRC, Adding ADD>
 __global__ void __launch_bounds__(kThreads, 2) equalize_formed_kernel(const FormedParams p, int groups) {
   extern __shared__ __align__(16) unsigned char smem[];
   using F = FormedShape<UP>;
-  using Lay = FormedEqLayout<UP, NRC>;
+  using Lay = FormedEqLayout<UP, NRC, ADD>;
   constexpr int NC = F::CA + NRC;
   const int U = p.s.U, NS = p.s.n_sym, C = p.s.Ceff, B = p.B, RS = formed_stride(B);
   const int k = blockIdx.x;
@@ -62,17 +78,54 @@ __global__ void __launch_bounds__(kThreads, 2) equalize_formed_kernel(const Form
   formed_wait();
 
   const int grp = threadIdx.x / F::GL, gl = threadIdx.x % F::GL, r = gl / 4, q = gl % 4;
-  if ((threadIdx.x & ~31) / F::GL >= groups) {   // whole warps without a group
+  const int first = (threadIdx.x & ~31) / F::GL;   // the warp's first group
+  const int parts = Lay::group_parts(C);           // more than one: groups == C, at_once
+  if (first >= groups * parts) {   // whole warps without a group
     if (at_once) __syncthreads();
+    if constexpr (ADD == kGroups) __syncthreads();
   } else {
     for (int c0 = 0; c0 < C; c0 += groups) {
-      const bool valid = grp < groups && c0 + grp < C;
-      const int c = valid ? c0 + grp : 0;
+      const int part = ADD == kGroups ? grp / groups : (grp >= groups), gc = grp - part * groups;   // part by part
+      const bool live = part < parts && c0 + gc < C;
+      const int c = live ? c0 + gc : 0;
       const int S = p.cl_uniform ? B / C : 0;
-      const int b0 = p.cl_uniform ? c * S : p.cl_off[c], b1 = p.cl_uniform ? b0 + S : p.cl_off[c + 1];
+      int b0 = p.cl_uniform ? c * S : p.cl_off[c], b1 = p.cl_uniform ? b0 + S : p.cl_off[c + 1];
+      if (ADD == kGroups && live) {
+        const int n = b1 - b0, a0 = b0;
+        b0 = a0 + part * n / parts;
+        b1 = a0 + (part + 1) * n / parts;
+      }
+      const int step = ADD == kSerial ? ((b1 - b0 + Lay::parts(C) - 1) / Lay::parts(C) + 1) & ~1 : 0;
       float re[F::RPL][NC], im[F::RPL][NC], rs[F::RPL];
-      formed_tile<UP, NRC, true, true>(Ws, RS, U, NS, b0, b1, r, q, valid, 0.f, re, im);
+      formed_tile<UP, NRC, true, true, ADD == kSerial>(Ws, RS, U, NS, b0, b1, r, q, live, 0.f, re, im, step);
       if (at_once) __syncthreads();   // one pass: the staged rows are no longer read
+      if constexpr (ADD == kGroups) {
+        // The other parts' tiles, added in order by the lanes of the first.
+        float* tiles = reinterpret_cast<float*>(areas + static_cast<size_t>(C) * Lay::AREA);
+        if (live && part > 0) {
+          float* t = tiles + static_cast<size_t>((part - 1) * C + c) * Lay::TILE * F::GL + gl;
+#pragma unroll
+          for (int i = 0; i < F::RPL; ++i)
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+              t[2 * (i * NC + j) * F::GL] = re[i][j];
+              t[(2 * (i * NC + j) + 1) * F::GL] = im[i][j];
+            }
+        }
+        __syncthreads();
+        if (first >= C) break;   // whole warps without a cluster of their own
+        for (int a = 1; a < parts && live && part == 0; ++a) {
+          const float* t = tiles + static_cast<size_t>((a - 1) * C + c) * Lay::TILE * F::GL + gl;
+#pragma unroll
+          for (int i = 0; i < F::RPL; ++i)
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+              re[i][j] += t[2 * (i * NC + j) * F::GL];
+              im[i][j] += t[(2 * (i * NC + j) + 1) * F::GL];
+            }
+        }
+      }
+      const bool valid = live && part == 0;
       unsigned zero_diag = 0;   // users this cluster cannot see (G_ii = 0), one bit per row of the lane
 #pragma unroll
       for (int i = 0; i < F::RPL; ++i) {
@@ -140,28 +193,44 @@ __global__ void __launch_bounds__(kThreads, 2) equalize_formed_kernel(const Form
   }
 }
 
-template <int UP, int NRC>
+template <int UP, int NRC, Adding ADD>
 cudaError_t launch_up(const FormedParams& p, cudaStream_t stream) {
-  using Lay = FormedEqLayout<UP, NRC>;
-  const size_t smem = Lay::bytes(p.B, p.s.U, p.s.n_sym, p.s.Ceff);
+  using Lay = FormedEqLayout<UP, NRC, ADD>;
+  const int C = p.s.Ceff;
+  const size_t smem = Lay::bytes(p.B, p.s.U, p.s.n_sym, C);
   static int configured[64] = {0};
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   if (dev < 64 && !configured[dev]) {
-    err = cudaFuncSetAttribute(equalize_formed_kernel<UP, NRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    err = cudaFuncSetAttribute(equalize_formed_kernel<UP, NRC, ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               227 * 1024);
     if (err != cudaSuccess) return err;
     configured[dev] = 1;
   }
-  equalize_formed_kernel<UP, NRC><<<p.s.n_sc, Lay::threads(p.B, p.s.Ceff), smem, stream>>>(p, Lay::groups(p.s.Ceff));
+  equalize_formed_kernel<UP, NRC, ADD><<<p.s.n_sc, Lay::threads(p.B, C), smem, stream>>>(p, Lay::groups(C));
   return cudaGetLastError();
+}
+
+// Parts in one lane where the sums fit its registers beside the part's tile (U = 16,
+// C = 2, S = 128, 1200 x 14: 91 us, groups 53) and its chains are short; groups where a
+// cluster has many antennas (U = 4, C = 2, 1200 x 1: S = 128 14.8 us, groups 12.1; S =
+// 16, 2000 x 1 5.7, groups 12.1) or an SM has at most two subcarriers (64 x 1: 3.9, 3.4).
+template <int UP, int NRC>
+cudaError_t launch_adding(const FormedParams& p, cudaStream_t stream) {
+  constexpr int kSms = 152;
+  if (p.s.Ceff > 4) return launch_up<UP, NRC, kOneChain>(p, stream);
+  if constexpr (kTileFloats<UP, NRC> <= 48) {
+    if (p.B < 64 * p.s.Ceff && p.s.n_sc > 2 * kSms) return launch_up<UP, NRC, kSerial>(p, stream);
+  }
+  return launch_up<UP, NRC, kGroups>(p, stream);
 }
 
 template <int UP>
 cudaError_t launch_nrc(const FormedParams& p, cudaStream_t stream) {
-  if (p.s.n_sym <= 4) return launch_up<UP, 1>(p, stream);
-  if (p.s.n_sym <= 8) return launch_up<UP, 2>(p, stream);
-  return launch_up<UP, 4>(p, stream);
+  if (p.s.n_sym <= 4) return launch_adding<UP, 1>(p, stream);
+  if (p.s.n_sym <= 8) return launch_adding<UP, 2>(p, stream);
+  return launch_adding<UP, 4>(p, stream);
 }
 
 }  // namespace
@@ -193,7 +262,7 @@ bool equalize_formed_fits(int precision, int B, int U, int n_sym, int C, int n_s
     return false;
   }
   const int UP = padded_users(U), NRC = n_sym <= 4 ? 1 : (n_sym <= 8 ? 2 : 4);
-  return 16 + formed_staged_bytes(B, U + n_sym) + static_cast<size_t>(C) * (4 * NRC * UP + UP / 2) * 8 <= 227 * 1024;   // bytes() at most
+  return 16 + formed_staged_bytes(B, U + n_sym) + static_cast<size_t>(C) * (4 * NRC * UP + UP / 2) * 8 <= 227 * 1024;   // bytes() at most (tiles: 41 KB)
 }
 
 cudaError_t launch_equalize_formed(const FormedParams& p, cudaStream_t stream) {

@@ -88,12 +88,14 @@ __device__ __forceinline__ void formed_wait() {
 // only the real parts (the same bits).  The training pair does the latter, so that
 // its X and G_b keep their bits: the gradient of the regularizers cancels 25- to
 // 45-fold over the subcarriers, and another rounding of the ill-conditioned solves
-// moves it by a few 1e-6 either way.
-template <int UP, int NRC, bool WITH_Y, bool HALF>
+// moves it by a few 1e-6 either way.  PARTS: every `part` antennas (even) are added up
+// by themselves first.
+template <int UP, int NRC, bool WITH_Y, bool HALF, bool PARTS = false>
 __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int NS, int b0, int b1, int r, int q,
                                             bool valid, float rho,
                                             float (&re)[FormedShape<UP>::RPL][FormedShape<UP>::CA + NRC],
-                                            float (&im)[FormedShape<UP>::RPL][FormedShape<UP>::CA + NRC]) {
+                                            float (&im)[FormedShape<UP>::RPL][FormedShape<UP>::CA + NRC],
+                                            int part = 0) {
   using F = FormedShape<UP>;
   constexpr int NC = F::CA + NRC, MC = WITH_Y ? NC : F::CA;
   const float* rowp[F::RPL];
@@ -113,15 +115,18 @@ __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int 
 #pragma unroll
     for (int j = 0; j < NC; ++j) re[i][j] = im[i][j] = 0.f;
   constexpr bool kHalf = F::RL == 4;
+  float pr[F::RPL][NC], pi[F::RPL][NC];   // PARTS: the part's sums
+  auto& ar = PARTS ? pr : re;
+  auto& ai = PARTS ? pi : im;
   auto acc = [&](int i, int j, float hr, float hi, float wr, float wi) {   // conj(h) w
     const bool far = kHalf && j < F::CA && j > i;
     if (HALF && far) return;
     if (!far) {
-      re[i][j] = fmaf(hr, wr, re[i][j]);
-      re[i][j] = fmaf(hi, wi, re[i][j]);
+      ar[i][j] = fmaf(hr, wr, ar[i][j]);
+      ar[i][j] = fmaf(hi, wi, ar[i][j]);
     }
-    im[i][j] = fmaf(hr, wi, im[i][j]);
-    im[i][j] = fmaf(-hi, wr, im[i][j]);
+    ai[i][j] = fmaf(hr, wi, ai[i][j]);
+    ai[i][j] = fmaf(-hi, wr, ai[i][j]);
   };
   auto single = [&](int b) {
     float2 h[F::RPL];
@@ -134,23 +139,42 @@ __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int 
       for (int i = 0; i < F::RPL; ++i) acc(i, j, h[i].x, h[i].y, w.x, w.y);
     }
   };
-  int b = b0, be = valid ? b1 : b0;
-  if ((b & 1) && b < be) single(b++);
-  for (; b + 1 < be; b += 2) {   // two antennas per 16-byte load
-    float4 h[F::RPL];
+  int b = b0;
+  const int b_end = valid ? b1 : b0;
+  do {
+    const int be = PARTS ? min((b + part) & ~1, b_end) : b_end;
+    if constexpr (PARTS) {
 #pragma unroll
-    for (int i = 0; i < F::RPL; ++i) h[i] = *reinterpret_cast<const float4*>(rowp[i] + 2 * b);
+      for (int i = 0; i < F::RPL; ++i)
 #pragma unroll
-    for (int j = 0; j < MC; ++j) {
-      const float4 w = *reinterpret_cast<const float4*>(colp[j] + 2 * b);
+        for (int j = 0; j < NC; ++j) pr[i][j] = pi[i][j] = 0.f;
+    }
+    if ((b & 1) && b < be) single(b++);
+    for (; b + 1 < be; b += 2) {   // two antennas per 16-byte load
+      float4 h[F::RPL];
 #pragma unroll
-      for (int i = 0; i < F::RPL; ++i) {
-        acc(i, j, h[i].x, h[i].y, w.x, w.y);
-        acc(i, j, h[i].z, h[i].w, w.z, w.w);
+      for (int i = 0; i < F::RPL; ++i) h[i] = *reinterpret_cast<const float4*>(rowp[i] + 2 * b);
+#pragma unroll
+      for (int j = 0; j < MC; ++j) {
+        const float4 w = *reinterpret_cast<const float4*>(colp[j] + 2 * b);
+#pragma unroll
+        for (int i = 0; i < F::RPL; ++i) {
+          acc(i, j, h[i].x, h[i].y, w.x, w.y);
+          acc(i, j, h[i].z, h[i].w, w.z, w.w);
+        }
       }
     }
-  }
-  if (b < be) single(b);
+    if (b < be) single(b++);
+    if constexpr (PARTS) {
+#pragma unroll
+      for (int i = 0; i < F::RPL; ++i)
+#pragma unroll
+        for (int j = 0; j < MC; ++j) {
+          re[i][j] += pr[i][j];
+          im[i][j] += pi[i][j];
+        }
+    }
+  } while (PARTS && b < b_end);
   if constexpr (kHalf) {
 #pragma unroll
     for (int i = 0; i < F::RPL; ++i) {
