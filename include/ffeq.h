@@ -81,7 +81,7 @@ typedef enum {
 typedef enum { FFEQ_PD = 0, FFEQ_FD = 1 } ffeq_arch;
 /* Arithmetic of the local preprocessing (G_c, y_c^MRC); the solve and fusion
  * are FP32 in every mode.  FP32, TF32X3 and FP16X3 problems may run one fused
- * FP32 kernel where it is the faster one (shapes 0 and 1 of the tuning below).
+ * FP32 kernel where it is the faster one (shape 0 of the tuning below).
  *   FFEQ_FP32    FP32 on the CUDA cores.
  *   FFEQ_TF32X3  tensor cores, each FP32 operand split into TF32 hi + lo, three
  *                products accumulated in FP32 (about FP32 accuracy).
@@ -202,9 +202,12 @@ ffeq_status ffeq_workspace_size(const ffeq_plan* plan, size_t* bytes);
  * N0 >= 0 and Es > 0 (finite).  workspace is a device buffer of at least
  * ffeq_workspace_size bytes; calls that share a workspace must be ordered on
  * one stream.  stream is a cudaStream_t (NULL = legacy default stream).
- * Asynchronous: returns after the launches (a contraction kernel, then a
- * solve/fusion kernel started by programmatic dependent launch); results are
- * ready when the stream reaches them. */
+ * Asynchronous: returns after the launches; results are ready when the stream
+ * reaches them.  A call is a contraction kernel, which fills the workspace as
+ * ffeq_local_preprocess does, then a solve/fusion kernel started by programmatic
+ * dependent launch (refinement adds its own); or one kernel that leaves the
+ * workspace untouched, where ffeq_plan_single_launch says so: ffeq_fuse_equalize
+ * must not follow such a call without ffeq_local_preprocess. */
 ffeq_status ffeq_equalize(const ffeq_plan* plan, const void* H, const void* y, float N0, float Es,
                           void* z, float* sigma2, float* llr, int* info,
                           void* workspace, size_t workspace_bytes, void* stream);
@@ -284,15 +287,17 @@ ffeq_status ffeq_fd_optimal_backward(const ffeq_plan* plan, const void* H, const
 
 /* Launch shape of a plan's contraction kernel (the arithmetic is that of the
  * plan's precision in every shape; with split-K (PD) the shapes differ in how
- * the antennas are split among warps, hence in summation order only):
- *   values[0]  0 = default (5 where it applies, else 1, 2 or 4 by the sizes),
+ * the antennas are split among warps, hence in summation order only; the one
+ * kernel of shape 0 below is FP32 for the split precisions too):
+ *   values[0]  0 = default (5 where it applies, else 1, 2 or 4 by the sizes);
+ *              with values[1] = 0, ffeq_equalize of an FD problem with FFEQ_LMMSE
+ *              or FFEQ_ZF, refine = 0 and FP32, TF32X3 or FP16X3 runs ONE kernel
+ *              that forms the local systems in FP32, solves, fuses and writes the
+ *              soft outputs (the workspace is left untouched) where that measured
+ *              faster: by U, n_sym, B, C and n_sc, FP32 mostly, the split
+ *              precisions with few users or symbols; ffeq_local_preprocess runs
+ *              the contraction;
  *              1 = 16 warps, one CTA per SM;
- *              in both, ffeq_equalize of an FD problem with FFEQ_LMMSE or FFEQ_ZF,
- *              refine = 0 and FP32, TF32X3 or FP16X3 runs ONE kernel that forms the
- *              local systems in FP32, solves, fuses and writes the soft outputs
- *              (the workspace is left untouched) where that measured faster: by
- *              U, n_sym, B, C and n_sc, FP32 mostly, the split precisions with
- *              few users or symbols; ffeq_local_preprocess runs the contraction;
  *              2 = 8 warps, two CTAs per SM (half the shared memory each),
  *              3 = BF16X3 only: each staged subcarrier converted once into BF16
  *                  hi/lo planes read with ldmatrix (needs B and B/C multiples of 4);
@@ -327,9 +332,16 @@ ffeq_status ffeq_fd_optimal_backward(const ffeq_plan* plan, const void* H, const
  * already queued on `stream`) and the graph's replay is timed with CUDA events,
  * so that host launch gaps do not decide the choice (eager calls where capture
  * is refused).  It keeps the fastest, makes `stream` wait for its work,
- * synchronizes, and must not run during stream capture. */
+ * synchronizes, and must not run during stream capture.  The one kernel of shape
+ * 0 is timed with them where the sizes allow it: if it is the fastest,
+ * ffeq_equalize keeps it until ffeq_plan_set_tuning, and the values are those of
+ * the fastest contraction, which ffeq_local_preprocess runs.
+ * ffeq_plan_single_launch writes 1 if ffeq_equalize of the plan is one kernel
+ * (shape 0 as above, autotuned or not, or shape 6 with 16-byte aligned device
+ * inputs), else 0. */
 ffeq_status ffeq_plan_set_tuning(ffeq_plan* plan, const int* values, int n);
 ffeq_status ffeq_plan_get_tuning(const ffeq_plan* plan, int* values, int n);
+ffeq_status ffeq_plan_single_launch(const ffeq_plan* plan, int* single);
 ffeq_status ffeq_plan_autotune(ffeq_plan* plan, const void* H, const void* y, float N0, float Es, void* z,
                                float* sigma2, float* llr, int* info, void* workspace, size_t workspace_bytes,
                                void* stream, int reps);

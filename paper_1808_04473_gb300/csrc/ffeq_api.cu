@@ -15,6 +15,7 @@ struct ffeq_plan {
   size_t workspace;      // bytes of the [n_sc][Ceff][U+n_sym][U] complex workspace
   int gram_variant = 0;  // contraction launch shape (0: default)
   int gram_stages = 0;   // staged units per CTA (0: as many as fit)
+  bool one_launch = false;   // autotuned: ffeq_equalize keeps the fused FP32 kernel, the shape above is the contraction's
   size_t off_X = 0, off_A = 0, off_F = 0;   // refinement arrays in the workspace
   ffeq::TensorMapCache* maps = nullptr;      // streamed contraction: encoded maps of recent inputs
   bool cl_uniform = true;                    // clusters of B / C antennas
@@ -393,14 +394,15 @@ ffeq_status ffeq_equalize(const ffeq_plan* plan, const void* H, const void* y, f
 
 namespace {
 
-// FP32, TF32x3 and FP16x3 FD problems of several clusters, in the default shape, are
-// equalized by the fused FP32 kernel where it is the faster one and a subcarrier
-// fits one CTA's shared memory (ffeq_formed.cu).
+// FP32, TF32x3 and FP16x3 FD problems of several clusters are equalized by the fused
+// FP32 kernel in the default shape, where it is the faster one and a subcarrier fits
+// one CTA's shared memory (ffeq_formed.cu), and where the autotuner found it faster
+// than every shape; a shape that the caller sets runs.
 bool formed_applies(const ffeq_plan* plan) {
   const ffeq_problem& p = plan->p;
   return p.refine == 0 &&
          (p.equalizer == FFEQ_LMMSE || p.equalizer == FFEQ_ZF) &&
-         (plan->gram_variant == ffeq::kGramAuto || plan->gram_variant == ffeq::kGram16) &&
+         (plan->one_launch || (plan->gram_variant == ffeq::kGramAuto && plan->gram_stages == 0)) &&
          ffeq::equalize_formed_fits(p.precision, p.B, p.U, p.n_sym, plan->Ceff, p.n_sc);
 }
 
@@ -670,6 +672,12 @@ ffeq_status ffeq_plan_get_tuning(const ffeq_plan* plan, int* values, int n) {
   return FFEQ_OK;
 }
 
+ffeq_status ffeq_plan_single_launch(const ffeq_plan* plan, int* single) {
+  if (!plan || !single) return FFEQ_ERR_INVALID_ARG;
+  *single = plan->gram_variant == ffeq::kGramFused || formed_applies(plan) ? 1 : 0;
+  return FFEQ_OK;
+}
+
 ffeq_status ffeq_plan_set_tuning(ffeq_plan* plan, const int* values, int n) {
   if (!plan || n != 2 || !values) return FFEQ_ERR_INVALID_ARG;
   if (values[0] < ffeq::kGramAuto || values[0] > ffeq::kGramVariantMax || values[1] < 0 ||
@@ -691,6 +699,7 @@ ffeq_status ffeq_plan_set_tuning(ffeq_plan* plan, const int* values, int n) {
     return FFEQ_ERR_UNSUPPORTED;
   plan->gram_variant = values[0];
   plan->gram_stages = values[1];
+  plan->one_launch = false;
   return FFEQ_OK;
 }
 
@@ -780,25 +789,36 @@ ffeq_status ffeq_plan_autotune_sets(ffeq_plan* plan, const void* const* H, const
     return cuda_fail(e);
   }
   const int old[2] = {plan->gram_variant, plan->gram_stages};
+  const bool old_one = plan->one_launch;
   float best = -1.f;
   int best_v[2] = {old[0], old[1]};
   ffeq_status s = FFEQ_OK;
+  // Time of a call with the plan as it stands (negative: not run), after one eager
+  // untimed call (first-use configuration happens outside capture).
+  auto timed = [&]() {
+    s = ffeq_equalize(plan, H[0], y[0], N0, Es, z, sigma2, llr, info, workspace, workspace_bytes, cs);
+    if (s != FFEQ_OK) return -1.f;
+    return time_equalize_calls(plan, H, y, n_sets, N0, Es, z, sigma2, llr, info, workspace, workspace_bytes, cs, reps,
+                               e0, e1, &s);
+  };
   for (int variant = ffeq::kGram16; variant <= ffeq::kGramVariantMax && s == FFEQ_OK; ++variant) {
     for (int stages = 1; stages <= 3 && s == FFEQ_OK; ++stages) {
       const int v[2] = {variant, stages};
       if (ffeq_plan_set_tuning(plan, v, 2) != FFEQ_OK) continue;
-      // One eager untimed call (first-use configuration happens outside capture).
-      s = ffeq_equalize(plan, H[0], y[0], N0, Es, z, sigma2, llr, info, workspace, workspace_bytes, cs);
-      if (s != FFEQ_OK) break;
-      const float ms = time_equalize_calls(plan, H, y, n_sets, N0, Es, z, sigma2, llr, info, workspace,
-                                           workspace_bytes, cs, reps, e0, e1, &s);
-      if (s != FFEQ_OK) break;
-      if (ms >= 0.f && (best < 0.f || ms < best)) {
+      const float ms = timed();
+      if (s == FFEQ_OK && ms >= 0.f && (best < 0.f || ms < best)) {
         best = ms;
         best_v[0] = variant;
         best_v[1] = stages;
       }
     }
+  }
+  // The fused FP32 kernel, which has no shape of its own.
+  plan->one_launch = true;
+  bool best_one = false;
+  if (s == FFEQ_OK && formed_applies(plan)) {
+    const float ms = timed();
+    best_one = s == FFEQ_OK && ms >= 0.f && (best < 0.f || ms < best);
   }
   // The caller's stream waits for everything run here.
   if (cudaEventRecord(dep, cs) == cudaSuccess) cudaStreamWaitEvent(st, dep, 0);
@@ -809,6 +829,7 @@ ffeq_status ffeq_plan_autotune_sets(ffeq_plan* plan, const void* const* H, const
   cudaStreamDestroy(cs);
   plan->gram_variant = s == FFEQ_OK ? best_v[0] : old[0];
   plan->gram_stages = s == FFEQ_OK ? best_v[1] : old[1];
+  plan->one_launch = s == FFEQ_OK ? best_one : old_one;
   return s;
 }
 

@@ -83,6 +83,7 @@ _SIGS = {
     "ffeq_device_status": ([ctypes.POINTER(_i), _i], _i),
     "ffeq_plan_set_tuning": ([_vp, ctypes.POINTER(_i), _i], _i),
     "ffeq_plan_get_tuning": ([_vp, ctypes.POINTER(_i), _i], _i),
+    "ffeq_plan_single_launch": ([_vp, ctypes.POINTER(_i)], _i),
     "ffeq_plan_autotune": ([_vp, _vp, _vp, _f, _f, _vp, _vp, _vp, _vp, _vp, _sz, _vp, _i], _i),
     "ffeq_plan_autotune_sets": ([_vp, ctypes.POINTER(_vp), ctypes.POINTER(_vp), _i, _f, _f, _vp, _vp, _vp, _vp, _vp,
                                  _sz, _vp, _i], _i),
@@ -275,6 +276,13 @@ def ffeq_plan_get_tuning(plan: Plan) -> tuple[int, int]:
     buf = (_i * 2)()
     _check("ffeq_plan_get_tuning", lib().ffeq_plan_get_tuning(plan.handle, buf, 2))
     return (buf[0], buf[1])
+
+
+def ffeq_plan_single_launch(plan: Plan) -> bool:
+    """Whether ffeq_equalize of the plan is one kernel; see include/ffeq.h."""
+    n = _i()
+    _check("ffeq_plan_single_launch", lib().ffeq_plan_single_launch(plan.handle, ctypes.byref(n)))
+    return bool(n.value)
 
 
 def ffeq_plan_autotune(plan: Plan, H, y, N0: float, Es: float, z, sigma2, llr=None, info=None, workspace=None,
