@@ -399,7 +399,15 @@ def soak(replay, seconds: float, torch):
 
 
 STEP_SHAPES = ((7, 0), (6, 0), (5, 0), (4, 0), (2, 0), (1, 0))   # launch shapes tried together for a whole step
-FUSED_SHAPE = 6          # the contraction and the solve in one launch (include/ffeq.h tuning)
+FUSED_SHAPE = 6          # the streamed contraction and the solve in one launch (include/ffeq.h tuning)
+
+
+def fused_kernel(ffeq, plan):
+    """The one kernel of a plan's ffeq_equalize on 16-byte aligned device inputs:
+    "streamed" (shape 6), "formed" (FP32) or None (a contraction, then a solve)."""
+    if not ffeq.ffeq_plan_single_launch(plan):
+        return None
+    return "streamed" if ffeq.ffeq_plan_get_tuning(plan)[0] == FUSED_SHAPE else "formed"
 
 
 def equalize_steps(R, shape, Hs, ys, N0, Es, *, precision, bits, K, warmup, equalizer=0, refine=0,
@@ -417,9 +425,10 @@ def equalize_steps(R, shape, Hs, ys, N0, Es, *, precision, bits, K, warmup, equa
     forked from and joined to the replay stream), so that one architecture's
     kernels can run while the other's hold fewer SMs.
     tune_step: after each plan's own autotuning, time the whole captured step for
-    every pair of contraction shapes in STEP_SHAPES, sequential and concurrent,
-    and keep the fastest (setup, outside the timed region): the best shape of a
-    plan alone is not always the best one next to the other plan's kernels.
+    every pair of contraction shapes in STEP_SHAPES (and the default shape where it
+    is one kernel of its own), sequential and concurrent, and keep the fastest
+    (setup, outside the timed region): the best shape of a plan alone is not always
+    the best one next to the other plan's kernels.
     tune_schedule: keep each plan's own tuning and choose only between the
     sequential and the concurrent step by timing both.
     Leaves the outputs of input set 0 in `outs`."""
@@ -504,8 +513,12 @@ def equalize_steps(R, shape, Hs, ys, N0, Es, *, precision, bits, K, warmup, equa
     schedule = {"concurrent": concurrent}
     if tune_step and not pinned:
         best = None
-        for tp in STEP_SHAPES:
-            for tf in STEP_SHAPES:
+        shapes = {}
+        for a in archs:
+            ffeq.ffeq_plan_set_tuning(plans[a], (0, 0))
+            shapes[a] = STEP_SHAPES + (((0, 0),) if ffeq.ffeq_plan_single_launch(plans[a]) else ())
+        for tp in shapes[archs[0]]:
+            for tf in shapes[archs[1]]:
                 try:
                     ffeq.ffeq_plan_set_tuning(plans[archs[0]], tp)
                     ffeq.ffeq_plan_set_tuning(plans[archs[1]], tf)
@@ -565,7 +578,7 @@ def equalize_steps(R, shape, Hs, ys, N0, Es, *, precision, bits, K, warmup, equa
     R.barrier()
     ms = start.elapsed_time(end)
     kern = {}
-    fused = {a: ffeq.ffeq_plan_get_tuning(plans[a])[0] == FUSED_SHAPE for a in archs}
+    fused = {a: fused_kernel(ffeq, plans[a]) for a in archs}
     if breakdown and split:
         # Each stage alone (with a fused plan, "local" and "fuse" are the separate
         # kernels the fused launch replaces, its contraction with a ring of 2),
@@ -1229,12 +1242,28 @@ def main():
                 "frac": achieved / FP32_ALU_TFLOPS, "traffic": traffic.get(f"{args.precision}:{name}"),
                 "algorithmic_flops_per_launch": flops, "kernel_ms": kern[name]}
 
+    def formed_roof(name):
+        # The one-launch FP32 kernel: contraction and solve on the CUDA cores.
+        clusters = C if name.startswith("fd") else 1
+        flops = (8 * B * (U * (U + 1) // 2 + U * n_sym) + solve_flops(U, n_sym, clusters)) * n_sc
+        achieved = flops / (kern[name] * 1e-3) / 1e12
+        return {"kernel": f"equalize_formed_kernel ({name[:2].upper()} local systems + solve + fusion + LLRs in FP32, "
+                          "one launch)", "bound": "alu", "achieved": achieved, "peak": FP32_ALU_TFLOPS,
+                "peak_source": "derived: 152 SM x 128 FP32 lanes x 2 flop x 2.07 GHz", "unit": "TFLOP/s",
+                "frac": achieved / FP32_ALU_TFLOPS, "traffic": traffic.get(f"{args.precision}:{name}"),
+                "algorithmic_flops_per_launch": flops, "kernel_ms": kern[name]}
+
     # The step's own kernels: a fused plan's one launch, else its two stages.
     step_kernels = []
     for tag, a in (("pd", ffeq.PD), ("fd", ffeq.FD)):
         step_kernels += [f"{tag}_fused"] if fused[a] else [f"{tag}_local", f"{tag}_fuse"]
     dom = max(step_kernels, key=kern.get)
-    roof = solve_roof(dom) if dom.endswith("_fuse") else gram_roof(dom)
+    if dom.endswith("_fuse"):
+        roof = solve_roof(dom)
+    elif dom.endswith("_fused") and fused[ffeq.PD if dom.startswith("pd") else ffeq.FD] == "formed":
+        roof = formed_roof(dom)
+    else:
+        roof = gram_roof(dom)
 
     gram_stage = {"pd": gram_roof("pd_local"), "fd": gram_roof("fd_local")}
     if "gram_stage_concurrent" in kern:
