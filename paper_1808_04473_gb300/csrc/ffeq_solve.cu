@@ -150,8 +150,8 @@ __device__ void batch_epilogue(const SolveParams& p, const float2* base, const i
 // denominators are g / A_uu; Es for MRC, whose are Es / sigma_c^2) and the LLRs.
 // System m's fusion area (numerators [n][UP], denominators) is areas + m stride.
 // Outputs are walked in the order (n, u), PADDED over u < UP, so that the index
-// splits by a constant, or over u < U (MRC, whose epilogue is most of its work: a
-// third of the lanes idle with U = 21 costs 6%).  zflag [spc][UP] (MRC, or
+// splits by a constant, or over u < U (few users of a padded group, and MRC, whose
+// epilogue is most of its work: a third of the lanes idle with U = 21 costs 6%).  zflag [spc][UP] (MRC, or
 // nullptr): users fused with the N0 -> 0 limit weights, whose variance is 0.
 template <int UP, bool PADDED>
 __device__ __forceinline__ void uniform_epilogue(const SolveParams& p, const float2* areas, int stride,
@@ -252,7 +252,10 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? (UP <= 16 ? 5 : 3) : 1) so
   }
   if (p.Xs) return;   // the refinement kernel fuses and writes the outputs
   __syncthreads();
-  uniform_epilogue<UP, true>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
+  // Half of the lanes would be idle over padded users (U = 4, 97 x 12, PD: a call of
+  // 13.8 us, 11.5 without padding).
+  if (2 * U <= UP) uniform_epilogue<UP, false>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
+  else uniform_epilogue<UP, true>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
 }
 
 template <int UP, int NRC, int MAXT>

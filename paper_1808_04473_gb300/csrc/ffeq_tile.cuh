@@ -70,15 +70,15 @@ __device__ __forceinline__ void tile_row_update(float (&re)[N], float (&im)[N], 
 // positive, or 0; rs[i] = 1 / p of row 4r + i.  Every lane of the warp must take
 // part (lanes past a 24-user group hold copies and change nothing else).
 template <int UP, int NRC>
-__device__ __forceinline__ int tile_sweep(float (&re)[4][UP / 4 + NRC], float (&im)[4][UP / 4 + NRC], int r, int q,
-                                          float (&rs)[4]) {
+__device__ __forceinline__ int tile_sweep(float (&re)[4][UP / 4 + NRC], float (&im)[4][UP / 4 + NRC], int U, int r,
+                                          int q, float (&rs)[4]) {
   using T = TileShape<UP, NRC>;
   constexpr int CA = T::CA, NC = T::NC, UN = T::UN, GL = T::GL;
   int fail = 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) rs[i] = 1.f;
 #pragma unroll 1
-  for (int t = 0; t < UP / UN; ++t) {
+  for (int t = 0; t < UP / UN && UN * t < U; ++t) {   // padding pivots change nothing
     static_for<UN>([&](auto sc) {
       constexpr int s = decltype(sc)::value;
       constexpr int I = s % 4, JC = s % CA;                    // the pivot's row and column in its tile
@@ -201,7 +201,7 @@ __device__ __forceinline__ int tile_solve_system(const float2* __restrict__ Dg, 
   };
   float rs[4] = {1.f, 1.f, 1.f, 1.f};
   if (Xs) cond = norm1(rs);
-  const int fail = tile_sweep<UP, NRC>(re, im, r, q, rs);
+  const int fail = tile_sweep<UP, NRC>(re, im, U, r, q, rs);
   if (Xs) {
     cond *= norm1(rs);
     if (valid && writer) {
