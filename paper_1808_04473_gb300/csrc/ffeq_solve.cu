@@ -146,17 +146,13 @@ __device__ void batch_epilogue(const SolveParams& p, const float2* base, const i
 
 // Outputs of a uniform problem, per subcarrier of this CTA: every (symbol, user)
 // sums the Ceff fusion numerators and denominators of its subcarrier and writes
-// z = num / den, sigma^2 = s2_scale / den (s2_scale = N0 for the solve, whose
-// denominators are g / A_uu; Es for MRC, whose are Es / sigma_c^2) and the LLRs.
+// z = num / den, sigma^2 = N0 / den (the denominators are g / A_uu) and the LLRs.
 // System m's fusion area (numerators [n][UP], denominators) is areas + m stride.
 // Outputs are walked in the order (n, u), PADDED over u < UP, so that the index
-// splits by a constant, or over u < U (few users of a padded group, and MRC, whose
-// epilogue is most of its work: a third of the lanes idle with U = 21 costs 6%).  zflag [spc][UP] (MRC, or
-// nullptr): users fused with the N0 -> 0 limit weights, whose variance is 0.
+// splits by a constant, or over u < U (few users of a padded group).
 template <int UP, bool PADDED>
 __device__ __forceinline__ void uniform_epilogue(const SolveParams& p, const float2* areas, int stride,
-                                                 const int* fail_sc, int sc0, int U, int NS, int Ceff, float s2_scale,
-                                                 const int* zflag = nullptr) {
+                                                 const int* fail_sc, int sc0, int U, int NS, int Ceff) {
   const int bits = p.llr_bits, hb = bits / 2;
   // (subcarrier s, output e) of this thread, advanced by the CTA's threads without
   // a division per output.
@@ -186,7 +182,7 @@ __device__ __forceinline__ void uniform_epilogue(const SolveParams& p, const flo
     } else if (dn > 0.f) {
       const float rr = rcp_approx(dn);
       zz = cscale(nm, rr);
-      s2 = (zflag && zflag[s * UP + u]) ? 0.f : s2_scale * rr;
+      s2 = p.N0 * rr;
     } else {
       zz = make_float2(0.f, 0.f);
       s2 = INFINITY;
@@ -254,8 +250,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? (UP <= 16 ? 5 : 3) : 1) so
   __syncthreads();
   // Half of the lanes would be idle over padded users (U = 4, 97 x 12, PD: a call of
   // 13.8 us, 11.5 without padding).
-  if (2 * U <= UP) uniform_epilogue<UP, false>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
-  else uniform_epilogue<UP, true>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff, p.N0);
+  if (2 * U <= UP) uniform_epilogue<UP, false>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff);
+  else uniform_epilogue<UP, true>(p, areas, Lay::kArea, fail_sc, sc0, U, NS, Ceff);
 }
 
 template <int UP, int NRC, int MAXT>
@@ -755,6 +751,44 @@ cudaError_t launch_full(const SolveParams& p, cudaStream_t stream) {
   return p.cond ? launch_full_as<UP, true>(p, stream) : launch_full_as<UP, false>(p, stream);
 }
 
+// Outputs of MRC, per subcarrier of this CTA, from the areas at base + system kMat:
+// z = num / den, sigma^2 = Es / den (0 for the users of zflag [spc][UP], fused with the
+// N0 -> 0 limit weights) and the LLRs.  A kernel that solves nothing is mostly this:
+// the walk and the wide LLR stores of uniform_epilogue cost calls up to 8% (U = 27, C =
+// 8, 111 x 13: 20.7 -> 22.3 us), their code being longer than a small grid repays.
+template <int UP>
+__device__ __forceinline__ void mrc_epilogue(const SolveParams& p, const float2* base, const int* zflag, int sc0, int U,
+                                             int NS, int Ceff) {
+  using Lay = SolveLayout<UP>;
+  const int spc = p.spc;
+  const int per = U * NS;   // uniform problem: every group has the problem's sizes
+  const int bits = p.llr_bits, hb = bits / 2;
+  for (int e = threadIdx.x; e < spc * per; e += blockDim.x) {
+    const int s = e / per, r = e - s * per;
+    const int n = r / U, u = r - n * U;
+    const int k = sc0 + s;
+    if (k >= p.n_sc) break;
+    float2 nm = make_float2(0.f, 0.f);
+    float dn = 0.f;
+    for (int cc = 0; cc < Ceff; ++cc) {
+      const float2* Lm = base + (s * Ceff + cc) * Lay::kMat + Lay::kRow;
+      nm = cadd(nm, Lm[n * UP + u]);
+      dn += reinterpret_cast<const float*>(Lm + Lay::kNum)[u];
+    }
+    float2 zz = make_float2(0.f, 0.f);
+    float s2 = INFINITY;
+    if (dn > 0.f) {
+      const float rr = rcp_approx(dn);
+      zz = cscale(nm, rr);
+      s2 = zflag[s * UP + u] ? 0.f : p.Es * rr;
+    }
+    const size_t zi = (static_cast<size_t>(k) * NS + n) * U + u;
+    p.z[zi] = zz;
+    if (n == 0) p.sigma2[static_cast<size_t>(k) * U + u] = s2;
+    if (bits) symbol_llr(zz, s2, p.llr_scale, hb, p.llr + zi * bits);
+  }
+}
+
 // Maximum-ratio combining (Sec. III-A) per (subcarrier, cluster), uniform
 // problems: lane i of a group of UP lanes reads row i of G_c and forms
 //   sigma_c^2 / Es = (rho G_ii + I_i) / G_ii^2,   I_i = sum_{j != i} |G_ij|^2,
@@ -772,7 +806,6 @@ template <int UP>
 __global__ void __launch_bounds__(512) mrc_fuse_kernel(const SolveParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Lay = SolveLayout<UP>;
-  int* fail_sc = reinterpret_cast<int*>(smem);
   float2* base = reinterpret_cast<float2*>(smem + 256);
   const int U = p.U, NS = p.n_sym, Ceff = p.Ceff;
   const int nmat = p.spc * Ceff;
@@ -780,7 +813,6 @@ __global__ void __launch_bounds__(512) mrc_fuse_kernel(const SolveParams p) {
   const int g = threadIdx.x / UP, i = threadIdx.x % UP;
   const int sc0 = blockIdx.x * p.spc;
   const bool noiseless = p.N0 == 0.f;
-  if (threadIdx.x < 64) fail_sc[threadIdx.x] = 0;
   for (int t = threadIdx.x; t < p.spc * UP; t += blockDim.x) zflag[t] = 0;
 
   // Wait for the contraction grid (programmatic dependent launch).
@@ -826,7 +858,7 @@ __global__ void __launch_bounds__(512) mrc_fuse_kernel(const SolveParams p) {
     Dn[i] = w;
   }
   __syncthreads();
-  uniform_epilogue<UP, false>(p, base + Lay::kRow, Lay::kMat, fail_sc, sc0, U, NS, Ceff, p.Es, zflag);
+  mrc_epilogue<UP>(p, base, zflag, sc0, U, NS, Ceff);
 }
 
 template <int UP>
