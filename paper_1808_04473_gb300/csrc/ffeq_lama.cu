@@ -144,39 +144,11 @@ __device__ __forceinline__ void lama_block(const LamaUnit& w, unsigned char* sme
 
   float2 s = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f), z;
   float phi = w.Es, tau;
-  for (int t = 1;; ++t) {
-    // z = y + s - G s + v.  A group lies within one warp: __syncwarp orders this
-    // iteration's stores before the loads, and the buffer written next iteration
-    // is the other one (the one after that is only written once every lane has
-    // passed the next __syncwarp, i.e. finished these loads).
-    z = yv;                 // t = 1: s = v = 0
-    if (t > 1) {
-      float* cur = (t & 1) ? sb1 : sb0;
-      cur[i] = s.x;
-      cur[UP + i] = s.y;
-      __syncwarp();
-      // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
-      // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
-      float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
-#pragma unroll
-      for (int j = 0; j < UP; j += 4) {
-        const float4 sr = *reinterpret_cast<const float4*>(cur + j);
-        const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
-          const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
-          rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
-          ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
-          ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
-          ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
-        }
-      }
-      const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
-      z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
-    }
-    tau = fmaf(beta, phi, n0n);
-    if (t >= w.iters) break;
+  // t = 1 has s = v = 0, so that z = y: an iteration of the loop is the denoiser of one
+  // t and the product of the next.
+  z = yv;
+  tau = fmaf(beta, phi, n0n);
+  for (int t = 1; t < w.iters; ++t) {
     const float inv_tau = rcp_approx(tau);
     const float l2t = kLog2e * inv_tau;
     float2 mean, var;
@@ -189,6 +161,34 @@ __device__ __forceinline__ void lama_block(const LamaUnit& w, unsigned char* sme
     v = __fmul2_rn(__fadd2_rn(z, make_float2(-s.x, -s.y)), make_float2(f, f));
     s = mean;
     phi = phin;
+    // z = y + s - G s + v.  A group lies within one warp: __syncwarp orders this
+    // iteration's stores before the loads, and the buffer written next iteration
+    // is the other one (the one after that is only written once every lane has
+    // passed the next __syncwarp, i.e. finished these loads).
+    float* cur = (t & 1) ? sb1 : sb0;
+    cur[i] = s.x;
+    cur[UP + i] = s.y;
+    __syncwarp();
+    // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
+    // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
+    float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
+#pragma unroll
+    for (int j = 0; j < UP; j += 4) {
+      const float4 sr = *reinterpret_cast<const float4*>(cur + j);
+      const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
+        const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
+        rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
+        ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
+        ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
+        ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
+      }
+    }
+    const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
+    z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
+    tau = fmaf(beta, phi, n0n);
   }
 
   if (g < ngroups) {
@@ -278,39 +278,11 @@ __global__ void __maxnreg__(UP == 32 ? 128 : 64) lama_kernel(const SolveParams p
 
   float2 s = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f), z;
   float phi = p.Es, tau;
-  for (int t = 1;; ++t) {
-    // z = y + s - G s + v.  A group lies within one warp: __syncwarp orders this
-    // iteration's stores before the loads, and the buffer written next iteration
-    // is the other one (the one after that is only written once every lane has
-    // passed the next __syncwarp, i.e. finished these loads).
-    z = yv;                 // t = 1: s = v = 0
-    if (t > 1) {
-      float* cur = (t & 1) ? sb1 : sb0;
-      cur[i] = s.x;
-      cur[UP + i] = s.y;
-      __syncwarp();
-      // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
-      // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
-      float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
-#pragma unroll
-      for (int j = 0; j < UP; j += 4) {
-        const float4 sr = *reinterpret_cast<const float4*>(cur + j);
-        const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
-          const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
-          rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
-          ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
-          ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
-          ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
-        }
-      }
-      const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
-      z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
-    }
-    tau = fmaf(beta, phi, n0n);
-    if (t >= p.lama_iters) break;
+  // t = 1 has s = v = 0, so that z = y: an iteration of the loop is the denoiser of one
+  // t and the product of the next.
+  z = yv;
+  tau = fmaf(beta, phi, n0n);
+  for (int t = 1; t < p.lama_iters; ++t) {
     const float inv_tau = rcp_approx(tau);
     const float l2t = kLog2e * inv_tau;
     float2 mean, var;
@@ -323,6 +295,34 @@ __global__ void __maxnreg__(UP == 32 ? 128 : 64) lama_kernel(const SolveParams p
     v = __fmul2_rn(__fadd2_rn(z, make_float2(-s.x, -s.y)), make_float2(f, f));
     s = mean;
     phi = phin;
+    // z = y + s - G s + v.  A group lies within one warp: __syncwarp orders this
+    // iteration's stores before the loads, and the buffer written next iteration
+    // is the other one (the one after that is only written once every lane has
+    // passed the next __syncwarp, i.e. finished these loads).
+    float* cur = (t & 1) ? sb1 : sb0;
+    cur[i] = s.x;
+    cur[UP + i] = s.y;
+    __syncwarp();
+    // (G s)_i = sum_j G_ij s_j: four paired partial sums over even / odd j,
+    // Re = sum g_re s_re - sum g_im s_im, Im = sum g_re s_im + sum g_im s_re.
+    float2 rr = make_float2(0.f, 0.f), ii = rr, ri = rr, ir = rr;
+#pragma unroll
+    for (int j = 0; j < UP; j += 4) {
+      const float4 sr = *reinterpret_cast<const float4*>(cur + j);
+      const float4 si = *reinterpret_cast<const float4*>(cur + UP + j);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 sr2 = h ? make_float2(sr.z, sr.w) : make_float2(sr.x, sr.y);
+        const float2 si2 = h ? make_float2(si.z, si.w) : make_float2(si.x, si.y);
+        rr = __ffma2_rn(gre[j / 2 + h], sr2, rr);
+        ii = __ffma2_rn(gim[j / 2 + h], si2, ii);
+        ri = __ffma2_rn(gre[j / 2 + h], si2, ri);
+        ir = __ffma2_rn(gim[j / 2 + h], sr2, ir);
+      }
+    }
+    const float2 gs = make_float2((rr.x + rr.y) - (ii.x + ii.y), (ri.x + ri.y) + (ir.x + ir.y));
+    z = __fadd2_rn(__fadd2_rn(__fadd2_rn(yv, s), make_float2(-gs.x, -gs.y)), v);
+    tau = fmaf(beta, phi, n0n);
   }
 
   if (g < ngroups) {
