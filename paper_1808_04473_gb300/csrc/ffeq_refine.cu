@@ -703,12 +703,21 @@ cudaError_t launch_tile(const RefineParams& p, cudaStream_t stream) {
                     RefineTileLayout(p.U, p.n_sym, p.max_S, NW).total, stream, p);
 }
 
+// Symbol rows of a lane by n_sym: with 16 symbols for 5 to 8 the padding outweighed
+// the tiles (PD, U = 20, B = 98, 2986 x 8: 202 us on the generic kernel, 210 on 16-symbol
+// tiles, 185 on 8).
 cudaError_t launch_tile_any(const RefineParams& p, cudaStream_t stream) {
-  const bool wide = p.n_sym > 4;
-  switch (padded_users(p.U)) {
-    case 8: return wide ? launch_tile<8, 4>(p, stream) : launch_tile<8, 1>(p, stream);
-    case 16: return wide ? launch_tile<16, 4>(p, stream) : launch_tile<16, 1>(p, stream);
-    default: return wide ? launch_tile<32, 4>(p, stream) : launch_tile<32, 1>(p, stream);
+  const int rhs = p.n_sym <= 4 ? 1 : (p.n_sym <= 8 ? 2 : 4);
+  switch (padded_users(p.U) * 10 + rhs) {
+    case 81: return launch_tile<8, 1>(p, stream);
+    case 82: return launch_tile<8, 2>(p, stream);
+    case 84: return launch_tile<8, 4>(p, stream);
+    case 161: return launch_tile<16, 1>(p, stream);
+    case 162: return launch_tile<16, 2>(p, stream);
+    case 164: return launch_tile<16, 4>(p, stream);
+    case 321: return launch_tile<32, 1>(p, stream);
+    case 322: return launch_tile<32, 2>(p, stream);
+    default: return launch_tile<32, 4>(p, stream);
   }
 }
 
