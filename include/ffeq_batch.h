@@ -120,6 +120,13 @@ int ffeq_batch_groups(const ffeq_batch* batch);
 ffeq_status ffeq_batch_get_tuning(const ffeq_batch* batch, int* values, int n);
 ffeq_status ffeq_batch_set_tuning(ffeq_batch* batch, const int* values, int n);
 
+/* How the library groups the batch, as 4 ints per group, min(n, 4 * groups) of
+ * them: {users padded, contraction shape (1: 16 warps, one CTA per SM; 2: 8
+ * warps, two CTAs per SM), most contraction stages, subcarriers}.  A tuning
+ * belongs to the grouping it was timed on; tunings kept elsewhere are keyed by
+ * it. */
+ffeq_status ffeq_batch_group_layout(const ffeq_batch* batch, int* values, int n);
+
 #ifdef __cplusplus
 }
 #endif

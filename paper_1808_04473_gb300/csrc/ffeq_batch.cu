@@ -431,6 +431,16 @@ ffeq_status ffeq_batch_get_tuning(const ffeq_batch* b, int* values, int n) {
   return FFEQ_OK;
 }
 
+ffeq_status ffeq_batch_group_layout(const ffeq_batch* b, int* values, int n) {
+  if (!b || (n > 0 && !values) || n < 0) return FFEQ_ERR_INVALID_ARG;
+  int w = 0;
+  for (const Group& g : b->groups) {
+    const int v[4] = {g.UP, g.variant, g.max_stages, static_cast<int>(std::min<long long>(g.n_units, 0x7fffffff))};
+    for (int t = 0; t < 4 && w < n; ++t) values[w++] = v[t];
+  }
+  return FFEQ_OK;
+}
+
 ffeq_status ffeq_batch_set_tuning(ffeq_batch* b, const int* values, int n) {
   if (!b || n != 4 * static_cast<int>(b->groups.size()) || (n > 0 && !values)) return FFEQ_ERR_INVALID_ARG;
   for (size_t gi = 0; gi < b->groups.size(); ++gi) {

@@ -95,6 +95,7 @@ _SIGS = {
     "ffeq_batch_equalize": ([_vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp], _i),
     "ffeq_batch_autotune": ([_vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp, _i], _i),
     "ffeq_batch_groups": ([_vp], _i),
+    "ffeq_batch_group_layout": ([_vp, ctypes.POINTER(_i), _i], _i),
     "ffeq_batch_get_tuning": ([_vp, ctypes.POINTER(_i), _i], _i),
     "ffeq_batch_set_tuning": ([_vp, ctypes.POINTER(_i), _i], _i),
 }
@@ -375,6 +376,14 @@ def ffeq_batch_get_tuning(batch: Batch) -> list[tuple[int, int, int, int]]:
     g = ffeq_batch_groups(batch)
     buf = (_i * max(1, 4 * g))()
     _check("ffeq_batch_get_tuning", lib().ffeq_batch_get_tuning(batch.handle, buf, 4 * g))
+    return [tuple(buf[4 * k:4 * k + 4]) for k in range(g)]
+
+
+def ffeq_batch_group_layout(batch: Batch) -> list[tuple[int, int, int, int]]:
+    """Per user group: (users padded, contraction shape, most contraction stages, subcarriers)."""
+    g = ffeq_batch_groups(batch)
+    buf = (_i * max(1, 4 * g))()
+    _check("ffeq_batch_group_layout", lib().ffeq_batch_group_layout(batch.handle, buf, 4 * g))
     return [tuple(buf[4 * k:4 * k + 4]) for k in range(g)]
 
 

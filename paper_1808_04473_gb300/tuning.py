@@ -2,9 +2,10 @@
 
 ``ffeq_batch_autotune`` times launch shapes on the GPU and keeps the fastest in
 the plan; this module stores the result in a JSON file keyed by the GPU name,
-the batch configuration and the multiset of instance shapes, so that a later
-process with the same batch skips the timing and restores the tuning with
-``ffeq_batch_set_tuning``.  Only launch shapes are cached: pipeline depth and
+the batch configuration, the multiset of instance shapes and the library's
+grouping of them, so that a later process with the same batch skips the timing
+and restores the tuning with ``ffeq_batch_set_tuning``, and one whose library
+groups the batch in another way (other contraction shapes) does not.  Only launch shapes are cached: pipeline depth and
 CTA width give bit-identical results, lanes per row changes only the rounding
 order of the solve.
 """
@@ -27,7 +28,8 @@ def default_cache_path() -> str:
 def batch_key(batch: ffeq.Batch, device_name: str) -> str:
     c = batch.config
     shapes = sorted((i.B, i.U, i.C, i.n_sc, i.n_sym) for i in batch.instances)
-    text = json.dumps([device_name, c.arch, c.precision, c.estimate, c.llr_bits, c.equalizer, c.lama_iters, shapes])
+    text = json.dumps([device_name, c.arch, c.precision, c.estimate, c.llr_bits, c.equalizer, c.lama_iters, shapes,
+                       ffeq.ffeq_batch_group_layout(batch)])
     return hashlib.sha256(text.encode()).hexdigest()[:32]
 
 
