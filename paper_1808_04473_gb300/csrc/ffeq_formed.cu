@@ -60,8 +60,10 @@ struct FormedEqLayout {
   }
 };
 
+// (Parts in one lane of eight users: 80 registers as in one chain; with more, fewer of
+// the small CTAs share an SM, U = 8, C = 2, S = 63, 800 x 4: 7.7 us, 11.1 without the cap.)
 template <int UP, int NRC, Adding ADD>
-__global__ void __launch_bounds__(kThreads, 2) equalize_formed_kernel(const FormedParams p, int groups) {
+__global__ void __launch_bounds__(kThreads, ADD == kSerial && UP == 8 && NRC < 4 ? 3 : 2) equalize_formed_kernel(const FormedParams p, int groups) {
   extern __shared__ __align__(16) unsigned char smem[];
   using F = FormedShape<UP>;
   using Lay = FormedEqLayout<UP, NRC, ADD>;

@@ -139,6 +139,20 @@ __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int 
       for (int i = 0; i < F::RPL; ++i) acc(i, j, h[i].x, h[i].y, w.x, w.y);
     }
   };
+  auto pair = [&](int b) {   // two antennas per 16-byte load
+    float4 h[F::RPL];
+#pragma unroll
+    for (int i = 0; i < F::RPL; ++i) h[i] = *reinterpret_cast<const float4*>(rowp[i] + 2 * b);
+#pragma unroll
+    for (int j = 0; j < MC; ++j) {
+      const float4 w = *reinterpret_cast<const float4*>(colp[j] + 2 * b);
+#pragma unroll
+      for (int i = 0; i < F::RPL; ++i) {
+        acc(i, j, h[i].x, h[i].y, w.x, w.y);
+        acc(i, j, h[i].z, h[i].w, w.z, w.w);
+      }
+    }
+  };
   int b = b0;
   const int b_end = valid ? b1 : b0;
   do {
@@ -150,19 +164,11 @@ __device__ __forceinline__ void formed_tile(const float* Ws, int RS, int U, int 
         for (int j = 0; j < NC; ++j) pr[i][j] = pi[i][j] = 0.f;
     }
     if ((b & 1) && b < be) single(b++);
-    for (; b + 1 < be; b += 2) {   // two antennas per 16-byte load
-      float4 h[F::RPL];
-#pragma unroll
-      for (int i = 0; i < F::RPL; ++i) h[i] = *reinterpret_cast<const float4*>(rowp[i] + 2 * b);
-#pragma unroll
-      for (int j = 0; j < MC; ++j) {
-        const float4 w = *reinterpret_cast<const float4*>(colp[j] + 2 * b);
-#pragma unroll
-        for (int i = 0; i < F::RPL; ++i) {
-          acc(i, j, h[i].x, h[i].y, w.x, w.y);
-          acc(i, j, h[i].z, h[i].w, w.z, w.w);
-        }
-      }
+    if constexpr (PARTS && NRC == 1) {
+#pragma unroll 2
+      for (; b + 1 < be; b += 2) pair(b);   // (a part is a few pairs)
+    } else {
+      for (; b + 1 < be; b += 2) pair(b);
     }
     if (b < be) single(b++);
     if constexpr (PARTS) {
