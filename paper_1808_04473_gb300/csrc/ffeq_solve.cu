@@ -814,6 +814,7 @@ __global__ void __launch_bounds__(512) mrc_fuse_kernel(const SolveParams p) {
   const int sc0 = blockIdx.x * p.spc;
   const bool noiseless = p.N0 == 0.f;
   for (int t = threadIdx.x; t < p.spc * UP; t += blockDim.x) zflag[t] = 0;
+  if (noiseless) __syncthreads();   // other warps set flags below
 
   // Wait for the contraction grid (programmatic dependent launch).
   asm volatile("griddepcontrol.wait;" ::: "memory");
