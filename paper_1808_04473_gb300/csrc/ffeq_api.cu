@@ -181,8 +181,7 @@ ffeq_status ffeq_plan_create_clusters(ffeq_plan** out, const ffeq_problem* p, co
   const int Ceff = p->arch == FFEQ_FD ? p->C : 1;
   if (ffeq::gram_stages(p->precision, p->B, p->U, p->n_sym, Ceff, false) < 1) return FFEQ_ERR_UNSUPPORTED;
   const int spc = ffeq::solve_subcarriers_per_cta(p->U, Ceff);
-  if (spc * Ceff * ffeq::padded_users(p->U) * (Ceff == 1 && ffeq::padded_users(p->U) == 16 ? 2 : 1) > 512 ||
-      ffeq::solve_smem_bytes(p->U, Ceff) > kSolveSmemLimit)
+  if (spc * Ceff * ffeq::padded_users(p->U) > 512 || ffeq::solve_smem_bytes(p->U, Ceff) > kSolveSmemLimit)
     return FFEQ_ERR_UNSUPPORTED;
   if (Ceff == 1) {
     uniform = true;          // PD sums every cluster: the partition does not enter (Eq. fullMRC)

@@ -28,7 +28,6 @@
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kSms = 152;
 constexpr int kMaxGroups = 64;                // queue counters in the first 256 bytes
 constexpr size_t kSolveSmemLimit = 227 * 1024;
 
@@ -80,7 +79,12 @@ struct ffeq_batch {
 
 namespace {
 
-// MRC runs one lane per row (no sweep); L-MMSE and ZF may split a row over two lanes.
+// Partial slot of an instance's split-K sums, sized for its group's padded users (the
+// kernel's slot stride).
+int slot_elems(const ffeq_instance& in) {
+  return ((in.U + in.n_sym) * (ffeq::padded_users(in.U) + 1) + 1) & ~1;
+}
+
 // Contraction shape of an instance: two CTAs of 8 warps per SM where one staged
 // unit fits half of the shared memory, so that one unit's waits, barriers and
 // reduction overlap the other's products (a CTA takes its units one at a time);
@@ -89,16 +93,16 @@ namespace {
 // BF16x3: FD 387 -> 342 us, PD 224 -> 168; FP32 FD 416 -> 377; 659 instances: 61 -> 54;
 // 326 instances: 42.6 with 16 warps, 43.8 with 8; 100: 53 and 56.
 int batch_variant(const ffeq_batch_config& cfg, const ffeq_instance& in, long long n_units) {
-  if (n_units < 3 * kSms) return ffeq::kGram16;
+  if (n_units < 3 * ffeq::kSms) return ffeq::kGram16;
   const int Ceff = cfg.arch == FFEQ_FD ? in.C : 1;
   const ffeq::GramCaps gc =
       ffeq::gram_instance_caps(cfg.precision, in.B, in.U, in.n_sym, Ceff, ffeq::kGram8x2);
-  const int slot = ((in.U + in.n_sym) * (ffeq::padded_users(in.U) + 1) + 1) & ~1;   // as in the groups below
-  const bool fits = ffeq::gram_stages_fit_bytes(gc.stage_elems, static_cast<size_t>(gc.slots) * slot * 8, true,
+  const bool fits = ffeq::gram_stages_fit_bytes(gc.stage_elems, static_cast<size_t>(gc.slots) * slot_elems(in) * 8, true,
                                                 ffeq::gram_smem_budget(ffeq::kGram8x2)) >= 1;
   return fits && cfg.precision != FFEQ_FP16X3 ? ffeq::kGram8x2 : ffeq::kGram16;   // FP16x3: the 16-warp shape only
 }
 
+// MRC runs one lane per row (no sweep); L-MMSE and ZF may split a row over two lanes.
 int lanes_per_row_default(int arch, int UP, int equalizer) {
   return (equalizer != FFEQ_MRC && equalizer != FFEQ_LAMA && arch == FFEQ_PD && UP == 16) ? 2 : 1;
 }
@@ -287,10 +291,8 @@ ffeq_status ffeq_batch_create(ffeq_batch** out, const ffeq_batch_config* cfg, co
       const ffeq::GramCaps gc = ffeq::gram_instance_caps(cfg->precision, inst[i].B, inst[i].U, inst[i].n_sym, Ceff,
                                                          variant);
       st[i] = gc.stage_elems;
-      sl[i] = gc.slot_elems;
       ns[i] = gc.slots;
-      // Slots are sized for the group's padded users (the kernel's slot stride).
-      sl[i] = ((inst[i].U + inst[i].n_sym) * (UP + 1) + 1) & ~1;
+      sl[i] = slot_elems(inst[i]);
     }
     // Instances without split-K partials first, then by decreasing staged size;
     // a group keeps the pipeline depth (up to 2) its first member allows alone.

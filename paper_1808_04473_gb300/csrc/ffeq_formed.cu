@@ -7,7 +7,9 @@
 // (Eq. fusionrule, Lemma 1; Thm. 3) and writes the outputs.  Neither the local
 // Gram matrices nor the matched filters go through the workspace, and the CUDA-core
 // contraction's staging, its partial sums and the second launch are gone.
-// What bounds it: the FMA pipe (the contraction and the sweep are about 60 / 40).
+// What bounds it: issue and its latencies (U = 16, C = 8, 1200 x 14: issue 56% of the
+// time, FMA pipe 43%, 11 warps per SM; one symbol, 8192 x 1: 74%, 44%, 15 warps; the
+// contraction and the sweep are about 60 / 40).
 #include <cmath>
 
 #include "ffeq_device.cuh"
@@ -220,7 +222,6 @@ cudaError_t launch_up(const FormedParams& p, cudaStream_t stream) {
 // 16, 2000 x 1 5.7, groups 12.1) or an SM has at most two subcarriers (64 x 1: 3.9, 3.4).
 template <int UP, int NRC>
 cudaError_t launch_adding(const FormedParams& p, cudaStream_t stream) {
-  constexpr int kSms = 152;
   if (p.s.Ceff > 4) return launch_up<UP, NRC, kOneChain>(p, stream);
   if constexpr (kTileFloats<UP, NRC> <= 48) {
     if (p.B < 64 * p.s.Ceff && p.s.n_sc > 2 * kSms) return launch_up<UP, NRC, kSerial>(p, stream);
@@ -237,25 +238,28 @@ cudaError_t launch_nrc(const FormedParams& p, cudaStream_t stream) {
 
 }  // namespace
 
-// Measured against the contraction and solve launches (us, before -> after): U = 4,
-// C = 2, S = 16, 2000 x 1: 38.8 -> 9.2; U = 8, C = 16, 3000 x 2: 112 -> 45; U = 15, C = 3,
-// S = 85, 1200 x 14: 127 -> 78; U = 16, C = 8, S = 32, 1200 x 14: 64.0 -> 61.4; U = 32,
-// C = 4, 1000 x 7: 162 -> 142.  Where it loses, the separate launches stay: tiles of 32
-// users with 16 right-hand sides spill registers (C = 16, 3300 x 14: 825 -> 1008), and
-// two or three clusters of 32 users leave too few warps per CTA for the contraction (C = 2,
-// S = 128, 300 x 14: 48 -> 72), as those of 16 users and 16 right-hand sides do where an
-// SM has less than two subcarriers (U = 16, C = 2, 64 x 14: 16.6 -> 20.6).
+// Measured against the contraction and solve launches (us a call, captured; before ->
+// after): U = 4, C = 2, S = 16, 2000 x 1: 36.1 -> 5.8; U = 8, C = 16, 3000 x 2: 110 -> 43;
+// U = 15, C = 3, S = 85, 1200 x 14: 126 -> 62; U = 16, C = 8, S = 32, 1200 x 14: 63.0 -> 59.2;
+// U = 32, C = 4, 1000 x 7: 160 -> 118.  Tiles of 32 users with 16 right-hand sides spill
+// registers and keep the separate launches (C = 16, 3300 x 14: 823 -> 1017), as do two
+// clusters of 24 users (1200 x 7: 101 -> 124).  Two to four clusters with few warps per CTA
+// were left out before their antennas were added in parts; with parts some of them would
+// gain (U = 16, C = 2, 64 x 14: 15.0 -> 11.4; U = 32, C = 2, 1200 x 4: 138 -> 111).
 //
 // TF32x3 and FP16x3 problems run here too where the tensor-core contraction and
 // the solve measured slower (FP32 is at least as accurate: every product rounds
 // once to 24 bits, and nothing is split).  BF16x3 does not: its results are its own.
-//   TF32x3: U = 16, C = 8, 1200 x 3: 56 -> 35; 1200 x 7: 59 -> 41; U = 10, 1200 x 14: 64 -> 47;
-//   U = 32, C = 8, 1200 x 3: 178 -> 133; not U = 14, C = 5, B = 250, 600 x 14 (37 -> 41).
-//   FP16x3: U = 12, C = 16, 800 x 8: 51 -> 37; U = 5, C = 2, 300 x 7: 23 -> 10; U = 11, C = 5,
-//   B = 120, 625 x 13: 33 -> 23; not U = 16, C = 8, 1200 x 14 (46 -> 62).
+//   TF32x3: U = 16, C = 8, 1200 x 3: 54 -> 30; 1200 x 7: 57 -> 38; U = 10, 1200 x 14: 67 -> 44;
+//   U = 32, C = 8, 1200 x 3: 176 -> 130; left out by an earlier measurement that a captured
+//   one does not bear out: U = 14, C = 5, B = 250, 600 x 14 (37.6 -> 33.4).
+//   FP16x3: U = 12, C = 16, 800 x 8: 56 -> 35; U = 5, C = 2, 300 x 7: 23 -> 6; U = 11, C = 5,
+//   B = 120, 625 x 13: 31 -> 21; U = 16, C = 8, 1200 x 8: 39.8 -> 39.2; not 1200 x 14 (44 -> 59),
+//   nor U = 20, C = 4, 600 x 4 (37 -> 49).
+// 260 random FD problems against shapes 1, 2 and 5: no problem taken here was faster there.
 bool equalize_formed_fits(int precision, int B, int U, int n_sym, int C, int n_sc) {
   if (C < 2 || (U > 16 && (n_sym > 8 || C < 4))) return false;
-  if (U > 8 && n_sym > 8 && C < 4 && n_sc < 2 * 152) return false;
+  if (U > 8 && n_sym > 8 && C < 4 && n_sc < 2 * kSms) return false;
   if (precision == FFEQ_TF32X3) {
     if (U > 16 ? n_sym > 4 : (U > 12 && n_sym > 8 && B > 128)) return false;
   } else if (precision == FFEQ_FP16X3) {

@@ -17,8 +17,9 @@
 // load phase reads in different banks, and natural rows stage with 16-byte
 // copies (4-byte ones before, to turn the rows around).  Measured on 8192
 // subcarriers, B = 128, U = 16, C = 8, one symbol (before -> after): training step
-// 407 -> 296 us (282 with HALF below), optimal adjoint 352 -> 292.  What
-// bounds them now: issue (72-74%), FMA pipe 39-48%, 16 warps per SM.
+// 407 -> 297 us (forward 175 -> 131, backward 211 -> 155; 282 in all with HALF below),
+// optimal adjoint 352 -> 292.  What bounds them now: issue (68-74%), FMA pipe 40-48%,
+// 16 warps per SM.
 //
 // Scalar FMAs: a paired FMA takes two cycles of the pipe (67 against 68 TFLOP/s
 // measured), so where the pipe is the limit the scalar form costs nothing and

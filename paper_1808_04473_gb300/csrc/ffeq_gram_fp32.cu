@@ -135,15 +135,14 @@ int gram_stages(int precision, int B, int U, int n_sym, int Ceff, bool bulk) {
 // small CTAs per SM where they fit and there are subcarriers enough for them,
 // because a CTA takes its subcarriers one at a time and its waits, barriers and
 // split-K reduction are exposed unless another CTA's products cover them.  Measured
-// (us a call, 16 warps -> this): PD TF32x3 U = 6, B = 96, 3000 x 4: 58 -> 27 (4 warps x 3);
-// PD TF32x3 U = 12, B = 100, 333 x 7: 20.6 -> 16.6 (4 x 3); FD BF16x3 U = 20, C = 5,
-// 800 x 6: 88 -> 78 (4 x 3, 10 of 16 warps busy before); PD TF32x3 U = 16, 1200 x 14: 55 -> 47
-// (8 x 2; 4 x 3 with one stage 49); PD FP32 U = 16, 1200 x 14: 60 -> 53 (8 x 2).  FD with
-// items for all 16 warps gains nothing (TF32x3 C = 8: 135 -> 136) and keeps them, as do
-// 100 subcarriers (14.3 -> 16.4) and, before 8 x 2 has two rounds for every CTA, 400
-// (PD TF32x3 U = 28: 51 -> 54).
+// (us a call, captured, 16 warps -> this): PD TF32x3 U = 6, B = 96, 3000 x 4: 55.7 -> 24.5 (4
+// warps x 3); PD TF32x3 U = 12, B = 100, 333 x 7: 18.5 -> 14.9 (4 x 3); FD BF16x3 U = 20, C =
+// 5, B = 200, 800 x 6: 79.5 -> 70.1 (4 x 3, 10 of 16 warps busy before); PD TF32x3 U = 16,
+// 1200 x 14: 52.5 -> 47.0 (8 x 2; 4 x 3 with one stage 48.5); PD FP32 U = 16, 1200 x 14: 57.9
+// -> 50.9 (8 x 2).  FD with items for all 16 warps gains nothing (TF32x3 C = 8, 1200 x 14:
+// 61.7 -> 63.2) and keeps them, as do 100 subcarriers (PD BF16x3 U = 12, 100 x 7: 12.0 ->
+// 14.8) and, before 8 x 2 has two rounds for every CTA, 400 (PD TF32x3 U = 28: 54.7 -> 56.8).
 static int default_shape(const GramParams& p, int precision) {
-  constexpr int kSms = 152;
   if (!p.bulk || p.n_sc < 2 * kSms || precision == FFEQ_FP16X3) return kGram16;
   auto stages_of = [&](int variant) {
     const GramCaps c = gram_instance_caps(precision, p.B, p.U, p.n_sym, p.Ceff, variant);

@@ -9,6 +9,8 @@
 
 namespace ffeq {
 
+constexpr int kSms = 152;   // streaming multiprocessors (where the dispatch rules draw their lines)
+
 constexpr int kNsymMax = 16;   // OFDM symbols per subcarrier held in registers
 constexpr int kMaxClusters = 64;   // FD clusters of a plan (the solve holds C * U padded <= 512 lanes)
 

@@ -291,7 +291,6 @@ cudaError_t launch_tile(const SolveParams& base, cudaStream_t stream) {
 // where every subcarrier has its own SM anyway, one wide CTA takes them at once.
 template <int UP, int NRC>
 cudaError_t launch_tile_nrc(const SolveParams& p, cudaStream_t stream) {
-  constexpr int kSms = 152;
   if (p.Ceff * TileShape<UP, NRC>::GL > 128 && p.n_sc <= kSms) return launch_tile<UP, NRC, 512>(p, stream);
   return launch_tile<UP, NRC, 128>(p, stream);
 }
@@ -996,15 +995,11 @@ cudaError_t launch_mrc_batch(const SolveParams& p, cudaStream_t stream) {
 
 // Subcarriers per CTA of the row kernel and of MRC, which a plan's limits count too
 // (the tile kernel takes its own): FD one, its C systems in one CTA with UP lanes
-// each; PD two where the users fill the lane group (one lane per row, measured
-// faster than two: half the instructions per system), else as many as made 128
-// lanes when a row of 9 to 15 users took two.
-static int lanes_per_row(int U, int Ceff) { return (Ceff == 1 && padded_users(U) == 16 && U != 16) ? 2 : 1; }
-
+// each; PD two where the users fill the lane group, else (MRC) CTAs of 64 or 128 lanes.
 int solve_subcarriers_per_cta(int U, int Ceff) {
   if (Ceff != 1) return 1;
   if (padded_users(U) == U) return 2;
-  return 128 / (padded_users(U) * lanes_per_row(U, Ceff));
+  return padded_users(U) == 8 ? 16 : 4;
 }
 
 size_t solve_smem_bytes(int U, int Ceff) {

@@ -11,13 +11,15 @@
 //   dL/drho_c = -sum_k Re tr(G_b^H X_c),  dL/dnu[c][u] = sum_k sum_n Re(conj(g_z,u,n) X_c,u,n)
 // (dX = M^{-1}(dB - dM X), dM = dH^H H + H^H dH + drho I, dB = dH^H Y + H^H dY.)
 // The factorization is recomputed in the backward pass (a Gauss-Jordan sweep on
-// [G_c + rho_c I | G_x,c]); the forward keeps the local Gram matrices and the
-// local estimates X_c in the workspace.
+// [G_c + rho_c I | G_x,c]); the forward keeps the local estimates X_c in the workspace.
 //
-// Every sweep is the paired-FMA Gauss-Jordan sweep with deferred scaling of
-// ffeq_gj.cuh on the augmented row [G_c + rho I | R] of UP + NR columns, NR the
-// right-hand-side columns rounded up from n_sym (4 when n_sym <= 4, else 16),
-// so a one-symbol problem does not sweep 16 columns of padding.
+// Two forms.  FP32 plans whose subcarrier fits in one CTA run the fused kernels, which
+// form the local Gram matrices as register tiles and sweep them there
+// (ffeq_formed.cuh).  The others run the contraction first, which leaves the Gram
+// matrices in the workspace, and the paired-FMA sweep of ffeq_gj.cuh on the augmented
+// row [G_c + rho I | R] of UP + NR columns, NR the right-hand-side columns rounded up
+// from n_sym (4 when n_sym <= 4, else 16), so a one-symbol problem does not sweep 16
+// columns of padding.
 //
 // Workspace: D [n_sc][C][U+n_sym][U] (contraction output, as ffeq_equalize),
 // X [n_sc][C][n_sym][U], Gb [n_sc][C][n_sym][U], W [n_sc][C][U][U] (complex) and
