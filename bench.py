@@ -1002,7 +1002,7 @@ def run_training(R, K, warmup):
     alg = n_sc * (24 * (B * U + B * n_sym) + 24 * U * n_sym)
     hbm_peak, peak_src = _peaks()
     achieved = alg / (ms / K * 1e-3) / 1e9
-    out["roofline"] = {"kernel": "whole step (contraction, train_forward, adjoint kernels)", "bound": "hbm",
+    out["roofline"] = {"kernel": "whole step (train_forward, train_backward and reduction kernels)", "bound": "hbm",
                        "achieved": achieved, "peak": hbm_peak, "peak_source": f"{peak_src} (STREAM-style copy)",
                        "unit": "GB/s", "frac": achieved / hbm_peak, "algorithmic_bytes_per_step": alg}
     # The FD estimate with the paper's optimal weights (ffeq_equalize) and its adjoint
@@ -1014,7 +1014,9 @@ def run_training(R, K, warmup):
     bws = torch.empty(bnb, dtype=torch.uint8, device=dev)
     zo = torch.empty_like(z)
     s2o = torch.empty((n_sc, U), dtype=torch.float32, device=dev)
-    ffeq.ffeq_plan_set_tuning(oplan, ffeq.ffeq_plan_get_tuning(plan))
+    # The tuned plan's choice: the values are a contraction's; the one-kernel form is the default's.
+    if not ffeq.ffeq_plan_single_launch(plan):
+        ffeq.ffeq_plan_set_tuning(oplan, ffeq.ffeq_plan_get_tuning(plan))
 
     def ostep(i):
         ffeq.ffeq_equalize(oplan, Hs[i], ys[i], p.N0, p.Es, zo, s2o, None, None, ows, onb, cap)

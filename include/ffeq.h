@@ -335,7 +335,8 @@ ffeq_status ffeq_fd_optimal_backward(const ffeq_plan* plan, const void* H, const
  * synchronizes, and must not run during stream capture.  The one kernel of shape
  * 0 is timed with them where the sizes allow it: if it is the fastest,
  * ffeq_equalize keeps it until ffeq_plan_set_tuning, and the values are those of
- * the fastest contraction, which ffeq_local_preprocess runs.
+ * the fastest contraction, which ffeq_local_preprocess runs.  Set on another
+ * plan, those values run that contraction; a plan left at {0, 0} runs the kernel.
  * ffeq_plan_single_launch writes 1 if ffeq_equalize of the plan is one kernel
  * (shape 0 as above, autotuned or not, or shape 6 with 16-byte aligned device
  * inputs), else 0. */
